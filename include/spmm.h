@@ -106,7 +106,8 @@ typedef struct {
                                 rows are then gathered one slab at a time, which keeps
                                 a slab of B resident in L2                              */
     int items_per_subwarp;   /* merge based: merge-path items (rows + nonzeros) per
-                                lane group; a tile holds 256 / lanes_per_row groups     */
+                                lane group; the tiles of a CTA hold 256 / lanes_per_row
+                                groups (128 / lanes_per_row up to 8 lanes)              */
     int long_row_len;        /* SPMM_ALG_ROW_SPLIT_HYBRID: rows with more nonzeros than
                                 this leave the row-block pass (queued rows of up to 4x
                                 this are taken by one lane group, with 4 or more lanes

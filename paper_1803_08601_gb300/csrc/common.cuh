@@ -1,6 +1,6 @@
 // Device-side building blocks shared by the SpMM kernels: element types and
-// 128-bit vector loads/stores, float32 accumulation helpers, and the bulk-copy
-// (TMA) / mbarrier primitives with bounded waits.
+// vector loads/stores of up to 128 bits, float32 accumulation helpers, and the
+// bulk-copy (TMA) / mbarrier primitives with bounded waits.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -14,11 +14,10 @@ namespace spmm {
 
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kThreads = 256;       // threads per CTA of the row-split, SDDMM and batched kernels
-// CTA shape of the merge-based kernel for W lanes per row: narrow rows (W <= 8)
-// use 128-thread CTAs with 1024-item tiles (small barrier domains, six CTAs per
-// SM); wide rows use 256-thread CTAs with 2048-item tiles (fewer tiles).
-__host__ __device__ constexpr int merge_cta_threads(int W) { return W >= 16 ? 256 : 128; }
-__host__ __device__ constexpr int merge_tile_items(int W) { return W >= 16 ? 2048 : 1024; }
+// Merge-based kernel of narrow rows (merge_kernel_narrow): 128-thread CTAs with
+// 1024-item tiles (small barrier domains, six CTAs per SM).
+constexpr int kNarrowThreads = 128;
+constexpr int kNarrowTile = 1024;
 constexpr int kUnroll = 8;     // gathers of B in flight per lane
 // Gathers in flight per lane for accesses of VEC elements of T: kUnroll for one
 // 16-byte vector, half as many for the two 16-byte vectors of the float32
@@ -85,9 +84,14 @@ __device__ __forceinline__ void load_vec(const T* p, float (&out)[VEC]) {
 // are accumulated, so a batch of 16-bit rows costs 4 registers per gather.
 template <typename T, int VEC> struct Raw;
 template <typename T> struct Raw<T, 1> { T v; };
+template <> struct Raw<float, 2> { float2 v; };
 template <> struct Raw<float, 4> { float4 v; };
 template <> struct Raw<float, 8> { float4 v, w; };  // two 16-byte vectors of one lane
+template <> struct Raw<__nv_bfloat16, 2> { uint32_t v; };
+template <> struct Raw<__nv_bfloat16, 4> { uint2 v; };
 template <> struct Raw<__nv_bfloat16, 8> { uint4 v; };
+template <> struct Raw<__half, 2> { uint32_t v; };
+template <> struct Raw<__half, 4> { uint2 v; };
 template <> struct Raw<__half, 8> { uint4 v; };
 
 template <typename T, int VEC>
@@ -98,10 +102,11 @@ __device__ __forceinline__ Raw<T, VEC> load_raw(const T* p) {
     } else if constexpr (sizeof(T) == 4 && VEC == 8) {
         r.v = __ldg(reinterpret_cast<const float4*>(p));
         r.w = __ldg(reinterpret_cast<const float4*>(p) + 1);
-    } else if constexpr (sizeof(T) == 4) {
+    } else if constexpr (sizeof(T) * VEC == 16 && sizeof(T) == 4) {
         r.v = __ldg(reinterpret_cast<const float4*>(p));
+    } else {
+        r.v = __ldg(reinterpret_cast<const decltype(r.v)*>(p));
     }
-    else r.v = __ldg(reinterpret_cast<const uint4*>(p));
     return r;
 }
 
@@ -113,10 +118,11 @@ __device__ __forceinline__ Raw<T, VEC> zero_raw() {
     } else if constexpr (sizeof(T) == 4 && VEC == 8) {
         r.v = make_float4(0.f, 0.f, 0.f, 0.f);
         r.w = r.v;
-    } else if constexpr (sizeof(T) == 4) {
+    } else if constexpr (sizeof(T) * VEC == 16 && sizeof(T) == 4) {
         r.v = make_float4(0.f, 0.f, 0.f, 0.f);
+    } else {
+        r.v = decltype(r.v){};
     }
-    else r.v = make_uint4(0u, 0u, 0u, 0u);
     return r;
 }
 
@@ -155,15 +161,28 @@ __device__ __forceinline__ void fma_raw(float (&acc)[VEC], float a, const Raw<T,
         acc[5] = fmaf(a, r.w.y, acc[5]);
         acc[6] = fmaf(a, r.w.z, acc[6]);
         acc[7] = fmaf(a, r.w.w, acc[7]);
+    } else if constexpr (sizeof(T) == 4 && VEC == 2) {
+        acc[0] = fmaf(a, r.v.x, acc[0]);
+        acc[1] = fmaf(a, r.v.y, acc[1]);
     } else if constexpr (sizeof(T) == 4) {
         acc[0] = fmaf(a, r.v.x, acc[0]);
         acc[1] = fmaf(a, r.v.y, acc[1]);
         acc[2] = fmaf(a, r.v.z, acc[2]);
         acc[3] = fmaf(a, r.v.w, acc[3]);
     } else {
-        const uint32_t w[4] = {r.v.x, r.v.y, r.v.z, r.v.w};
+        uint32_t w[VEC / 2];
+        if constexpr (VEC == 2) {
+            w[0] = r.v;
+        } else {
+            w[0] = r.v.x;
+            w[1] = r.v.y;
+            if constexpr (VEC == 8) {
+                w[2] = r.v.z;
+                w[3] = r.v.w;
+            }
+        }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < VEC / 2; ++i) {
             acc[2 * i] = fmaf(a, Elem<T>::to_f(Elem<T>::from_bits((uint16_t)(w[i] & 0xffffu))), acc[2 * i]);
             acc[2 * i + 1] = fmaf(a, Elem<T>::to_f(Elem<T>::from_bits((uint16_t)(w[i] >> 16))), acc[2 * i + 1]);
         }
@@ -216,11 +235,13 @@ __device__ __forceinline__ void accum_raw(float (&acc)[VEC], float a, const Raw<
     }
 }
 
-// Store VEC floats as TC at p (p aligned to VEC * sizeof(TC) when VEC > 1).
+// Store VEC floats as TC at p (p aligned to min(VEC * sizeof(TC), 16) bytes when VEC > 1).
 template <typename TC, int VEC>
 __device__ __forceinline__ void store_vec(TC* p, const float (&v)[VEC]) {
     if constexpr (VEC == 1) {
         p[0] = Elem<TC>::from_f(v[0]);
+    } else if constexpr (sizeof(TC) == 4 && VEC == 2) {
+        *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
     } else if constexpr (sizeof(TC) == 4) {
 #pragma unroll
         for (int i = 0; i < VEC; i += 4)
@@ -236,9 +257,11 @@ __device__ __forceinline__ void store_vec(TC* p, const float (&v)[VEC]) {
         }
         if constexpr (VEC == 8) {
             *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-        } else {
-            static_assert(VEC == 4, "unexpected vector width");
+        } else if constexpr (VEC == 4) {
             *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
+        } else {
+            static_assert(VEC == 2, "unexpected vector width");
+            *reinterpret_cast<uint32_t*>(p) = w[0];
         }
     }
 }

@@ -469,7 +469,7 @@ __device__ __forceinline__ void merge_tile(const MergeArgs& a, const MergeView<T
 // and returns.
 template <typename TV, typename TB, typename TC, int VEC, int W, typename SR = PlusTimes>
 __device__ __forceinline__ void merge_kernel_body(const MergeArgs& a) {
-    constexpr int NT = merge_cta_threads(W);
+    constexpr int NT = kNarrowThreads;
     extern __shared__ __align__(128) unsigned char smem[];
     MergeView<TV, VEC, W, NT> v{smem, a.ips};
     pdl_wait();               // the partition (launched just before) has finished writing limits
@@ -520,15 +520,10 @@ __device__ __forceinline__ void merge_kernel_body(const MergeArgs& a) {
     }
 }
 
-// Narrow rows (W <= 8): 128-thread CTAs, six per SM.
+// Narrow rows (W <= 8): six CTAs per SM.  Wider ones, and narrow ones of longer
+// rows, run merge_kernel (merge.cuh); merge_narrow (spmm_api.cu) has the line.
 template <typename TV, typename TB, typename TC, int VEC, int W, typename SR = PlusTimes>
-__global__ void __launch_bounds__(128, 6) merge_kernel_narrow(MergeArgs a) {
-    merge_kernel_body<TV, TB, TC, VEC, W, SR>(a);
-}
-
-// Wide rows (W >= 16): 256-thread CTAs.
-template <typename TV, typename TB, typename TC, int VEC, int W, typename SR = PlusTimes>
-__global__ void __launch_bounds__(256) merge_kernel_wide(MergeArgs a) {
+__global__ void __launch_bounds__(kNarrowThreads, 6) merge_kernel_narrow(MergeArgs a) {
     merge_kernel_body<TV, TB, TC, VEC, W, SR>(a);
 }
 

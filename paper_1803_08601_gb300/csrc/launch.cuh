@@ -8,15 +8,19 @@
 
 #include "hybrid.cuh"
 #include "kernels.cuh"
+#include "merge.cuh"
 
 namespace spmm {
 
 // Launch shape chosen by the host: vec = elements per lane access (1 or the
-// 16-byte width of B's type), W = lanes per row, slabs = column slabs,
-// ips = merge-path items per lane group.
+// 16-byte width of B's type; merge based: any power of two up to it), W =
+// lanes per row, chunks = column chunks of W * vec columns that a lane group
+// covers together (merge based; 1 elsewhere), slabs = column slabs, ips =
+// merge-path items per lane group of merge_kernel_narrow (0: merge_kernel).
 struct Shape {
     int vec;
     int W;
+    int chunks;
     int slabs;
     int ips;
 };
@@ -25,8 +29,7 @@ extern std::atomic<long long> g_launches;
 
 using RowSplitFn = cudaError_t (*)(const RowSplitArgs&, const Shape&, cudaStream_t);
 using MergeFn = cudaError_t (*)(const MergeArgs&, const Shape&, int grid_cap, cudaStream_t);
-using MergeSmemFn = size_t (*)(const Shape&);
-using FixupFn = cudaError_t (*)(const MergeArgs&, cudaStream_t);
+using FixupFn = cudaError_t (*)(const MergeArgs&, int tiles, cudaStream_t);
 using SpmvRowSplitFn = cudaError_t (*)(const RowSplitArgs&, int lanes, cudaStream_t);
 using SpmvMergeFn = cudaError_t (*)(const MergeArgs&, int items_per_thread, cudaStream_t);
 using TiledFn = cudaError_t (*)(const TiledArgs&, const Shape&, cudaStream_t);
@@ -35,7 +38,6 @@ using RowSplitHybridFn = cudaError_t (*)(const RowSplitArgs&, const LongRowArgs&
 struct Launchers {
     RowSplitFn rowsplit;
     MergeFn merge;
-    MergeSmemFn merge_smem;
     FixupFn fixup;
     SpmvRowSplitFn spmv_rowsplit;  // n = 1
     SpmvMergeFn spmv_merge;        // n = 1, tiles of kThreads * items_per_thread items (4, 8 or 16)
@@ -160,14 +162,10 @@ cudaError_t hybrid_launch(const RowSplitArgs& a, const LongRowArgs& l, const Sha
 }
 
 template <typename TV, typename TB, typename TC, int VEC, int W, typename SR>
-cudaError_t merge_launch_one(const MergeArgs& a, const Shape& s, int grid_cap, cudaStream_t st) {
-    constexpr int NT = merge_cta_threads(W);
+cudaError_t merge_narrow_launch_one(const MergeArgs& a, const Shape& s, int grid_cap, cudaStream_t st) {
+    constexpr int NT = kNarrowThreads;
     using L = MergeSmem<TV, VEC, W, NT>;
-    auto kern = [] {
-        if constexpr (NT == 256) return merge_kernel_wide<TV, TB, TC, VEC, W, SR>;
-        else return merge_kernel_narrow<TV, TB, TC, VEC, W, SR>;
-    }();
-    static_assert(NT == 128 || NT == 256, "merge CTA shapes");
+    auto kern = merge_kernel_narrow<TV, TB, TC, VEC, W, SR>;
     const size_t smem = L::total(s.ips);
     // per-instantiation cache of the opt-in shared-memory size and occupancy
     static thread_local int cached_dev = -1;
@@ -207,31 +205,78 @@ cudaError_t merge_launch_one(const MergeArgs& a, const Shape& s, int grid_cap, c
 }
 
 template <typename TV, typename TB, typename TC, int VEC, typename SR>
-cudaError_t merge_launch_vec(const MergeArgs& a, const Shape& s, int grid_cap, cudaStream_t st) {
+cudaError_t merge_narrow_launch(const MergeArgs& a, const Shape& s, int grid_cap, cudaStream_t st) {
     switch (s.W) {
-        case 1: return merge_launch_one<TV, TB, TC, VEC, 1, SR>(a, s, grid_cap, st);
-        case 2: return merge_launch_one<TV, TB, TC, VEC, 2, SR>(a, s, grid_cap, st);
-        case 4: return merge_launch_one<TV, TB, TC, VEC, 4, SR>(a, s, grid_cap, st);
-        case 8: return merge_launch_one<TV, TB, TC, VEC, 8, SR>(a, s, grid_cap, st);
-        case 16: return merge_launch_one<TV, TB, TC, VEC, 16, SR>(a, s, grid_cap, st);
-        case 32: return merge_launch_one<TV, TB, TC, VEC, 32, SR>(a, s, grid_cap, st);
+        case 1: return merge_narrow_launch_one<TV, TB, TC, VEC, 1, SR>(a, s, grid_cap, st);
+        case 2: return merge_narrow_launch_one<TV, TB, TC, VEC, 2, SR>(a, s, grid_cap, st);
+        case 4: return merge_narrow_launch_one<TV, TB, TC, VEC, 4, SR>(a, s, grid_cap, st);
+        case 8: return merge_narrow_launch_one<TV, TB, TC, VEC, 8, SR>(a, s, grid_cap, st);
         default: return cudaErrorInvalidValue;
     }
 }
 
+// Merge compute: a warp per tile (a.num_tiles of them), slab by slab, chained
+// behind the partition with programmatic dependent launch.
+template <typename TV, typename TB, typename TC, int VEC, int E, int W, typename SR>
+cudaError_t merge_launch_one(const MergeArgs& a, const Shape& s, cudaStream_t st) {
+    if (a.num_tiles < 1) return cudaSuccess;
+    if (s.slabs < 1 || s.slabs > 65535) return cudaErrorInvalidConfiguration;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((long long)a.num_tiles + kMergeWarps - 1) / kMergeWarps), (unsigned)s.slabs);
+    cfg.blockDim = dim3(kMergeThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // overlap the partition's tail
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, merge_kernel<TV, TB, TC, VEC, E, W, SR>, a);
+    if (e == cudaSuccess) e = cudaGetLastError();
+    if (e == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
+    return e;
+}
+
+// The shapes merge_shape (spmm_api.cu) picks: 16-byte accesses, or narrower
+// ones, from 33 columns on with 32 lanes and up to 4 chunks.
 template <typename TV, typename TB, typename TC, typename SR>
 cudaError_t merge_launch(const MergeArgs& a, const Shape& s, int grid_cap, cudaStream_t st) {
     constexpr int V = Elem<TB>::kVec;
-    return s.vec == 1 ? merge_launch_vec<TV, TB, TC, 1, SR>(a, s, grid_cap, st)
-                      : merge_launch_vec<TV, TB, TC, V, SR>(a, s, grid_cap, st);
+    if (s.ips > 0)
+        return s.vec == 1 ? merge_narrow_launch<TV, TB, TC, 1, SR>(a, s, grid_cap, st)
+                          : merge_narrow_launch<TV, TB, TC, V, SR>(a, s, grid_cap, st);
+    if (s.vec == V) {
+        switch (s.W) {
+            case 8: return merge_launch_one<TV, TB, TC, V, 1, 8, SR>(a, s, st);
+            case 16: return merge_launch_one<TV, TB, TC, V, 1, 16, SR>(a, s, st);
+            case 32: return merge_launch_one<TV, TB, TC, V, 1, 32, SR>(a, s, st);
+            default: return cudaErrorInvalidValue;
+        }
+    }
+    if (s.vec == 2 && s.W == 32)
+        return s.chunks == 2 ? merge_launch_one<TV, TB, TC, 2, 2, 32, SR>(a, s, st)
+                             : merge_launch_one<TV, TB, TC, 2, 1, 32, SR>(a, s, st);
+    if (s.vec != 1) return cudaErrorInvalidValue;
+    switch (s.W) {
+        case 1: return merge_launch_one<TV, TB, TC, 1, 1, 1, SR>(a, s, st);
+        case 2: return merge_launch_one<TV, TB, TC, 1, 1, 2, SR>(a, s, st);
+        case 4: return merge_launch_one<TV, TB, TC, 1, 1, 4, SR>(a, s, st);
+        case 8: return merge_launch_one<TV, TB, TC, 1, 1, 8, SR>(a, s, st);
+        case 16: return merge_launch_one<TV, TB, TC, 1, 1, 16, SR>(a, s, st);
+        case 32:
+            return s.chunks == 4   ? merge_launch_one<TV, TB, TC, 1, 4, 32, SR>(a, s, st)
+                   : s.chunks == 2 ? merge_launch_one<TV, TB, TC, 1, 2, 32, SR>(a, s, st)
+                                   : merge_launch_one<TV, TB, TC, 1, 1, 32, SR>(a, s, st);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
-// FIXCARRYOUT launch: a warp per tile (grid-stride), chained behind the merge
-// kernel with programmatic dependent launch.
+// FIXCARRYOUT launch over the `tiles` entries of carry_row / head_row: a warp
+// per entry (grid-stride), chained behind the merge kernel with programmatic
+// dependent launch.
 template <typename TC, typename SR>
-cudaError_t fixup_launch(const MergeArgs& ma, cudaStream_t st) {
+cudaError_t fixup_launch(const MergeArgs& ma, int tiles, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min<long long>(((long long)ma.num_tiles + 7) / 8, 152LL * 8));
+    cfg.gridDim = dim3((unsigned)std::min<long long>(((long long)tiles + 7) / 8, 152LL * 8));
     cfg.blockDim = dim3(256);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
@@ -241,7 +286,7 @@ cudaError_t fixup_launch(const MergeArgs& ma, cudaStream_t st) {
     cfg.numAttrs = 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, merge_fixup_kernel<TC, SR>, (const int*)ma.carry_row,
                                        (const int*)ma.head_row, (const float*)ma.carry, (const float*)ma.head,
-                                       ma.num_tiles, ma.n, static_cast<TC*>(ma.C), ma.ldc, ma.status);
+                                       tiles, ma.n, static_cast<TC*>(ma.C), ma.ldc, ma.status);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
     return e;
@@ -334,28 +379,21 @@ cudaError_t tiled_launch(const TiledArgs& a, const Shape& s, cudaStream_t st) {
     }
 }
 
+// Dynamic shared memory of merge_kernel_narrow.
 template <typename TV, int VEC>
 size_t merge_smem_vec(const Shape& s) {
     switch (s.W) {
-        case 1: return MergeSmem<TV, VEC, 1, merge_cta_threads(1)>::total(s.ips);
-        case 2: return MergeSmem<TV, VEC, 2, merge_cta_threads(2)>::total(s.ips);
-        case 4: return MergeSmem<TV, VEC, 4, merge_cta_threads(4)>::total(s.ips);
-        case 8: return MergeSmem<TV, VEC, 8, merge_cta_threads(8)>::total(s.ips);
-        case 16: return MergeSmem<TV, VEC, 16, merge_cta_threads(16)>::total(s.ips);
-        default: return MergeSmem<TV, VEC, 32, merge_cta_threads(32)>::total(s.ips);
+        case 1: return MergeSmem<TV, VEC, 1, kNarrowThreads>::total(s.ips);
+        case 2: return MergeSmem<TV, VEC, 2, kNarrowThreads>::total(s.ips);
+        case 4: return MergeSmem<TV, VEC, 4, kNarrowThreads>::total(s.ips);
+        default: return MergeSmem<TV, VEC, 8, kNarrowThreads>::total(s.ips);
     }
-}
-
-template <typename TV, typename TB, typename TC>
-size_t merge_smem(const Shape& s) {
-    constexpr int V = Elem<TB>::kVec;
-    return s.vec == 1 ? merge_smem_vec<TV, 1>(s) : merge_smem_vec<TV, V>(s);
 }
 
 template <typename TV, typename TB, typename TC, typename SR = PlusTimes>
 Launchers make_launchers() {
-    return Launchers{&rowsplit_launch<TV, TB, TC, SR>, &merge_launch<TV, TB, TC, SR>, &merge_smem<TV, TB, TC>,
-                     &fixup_launch<TC, SR>, &spmv_rowsplit_launch<TV, TB, TC, SR>, &spmv_merge_launch<TV, TB, TC, SR>,
+    return Launchers{&rowsplit_launch<TV, TB, TC, SR>, &merge_launch<TV, TB, TC, SR>, &fixup_launch<TC, SR>,
+                     &spmv_rowsplit_launch<TV, TB, TC, SR>, &spmv_merge_launch<TV, TB, TC, SR>,
                      &tiled_launch<TV, TB, TC, SR>, &hybrid_launch<TV, TB, TC, SR>};
 }
 

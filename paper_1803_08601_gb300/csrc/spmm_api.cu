@@ -72,7 +72,7 @@ namespace {
 
 constexpr double kPaperThreshold = 9.35;  // Section 5.4
 constexpr unsigned long long kWaitLimitNs = 1000000000ull;  // 1 s per bounded wait
-constexpr size_t kMaxSmem = 200 * 1024;  // dynamic shared memory the merge kernel may request
+constexpr size_t kMaxSmem = 200 * 1024;  // dynamic shared memory merge_kernel_narrow may request
 
 struct TypeCombo {
     int tv, tb, tc;
@@ -151,23 +151,22 @@ bool shape_for(int n, int vec, const spmm_tuning_t* t, Shape* s) {
         W = pow2_ceil(chunks);
     }
     s->W = W;
+    s->chunks = 1;
     s->slabs = (int)((chunks + W - 1) / W);
-    if (s->slabs > 65535) return false;
-    const int groups = merge_cta_threads(W) / W;  // lane groups per merge CTA
-    int ips = (t && t->items_per_subwarp > 0) ? t->items_per_subwarp : merge_tile_items(W) / groups;
-    if (ips < 4) ips = 4;
-    if (ips > 4096) ips = 4096;
-    s->ips = ips;
-    return true;
+    return s->slabs <= 65535;
 }
 
-// 16-byte accesses when n, both leading dimensions and both base pointers allow them.
+// vec elements per access of B and of C: n, both leading dimensions and both base pointers allow them.
+bool access_ok(int vec, int n, int tb, int tc, const void* B, long long ldb, const void* C, long long ldc) {
+    return n % vec == 0 && ldb % vec == 0 && ldc % vec == 0 && ((uintptr_t)B % (uintptr_t)(vec * dtype_size(tb))) == 0 &&
+           ((uintptr_t)C % (uintptr_t)(vec * dtype_size(tc))) == 0;
+}
+
+// 16-byte accesses when they are aligned.
 bool choose_shape(int n, int tb, int tc, const void* B, long long ldb, const void* C, long long ldc,
                   const spmm_tuning_t* t, Shape* s) {
     const int V = 16 / dtype_size(tb);
-    const bool vec_ok = n % V == 0 && ldb % V == 0 && ldc % V == 0 && ((uintptr_t)B % 16) == 0 &&
-                        ((uintptr_t)C % (uintptr_t)(V * dtype_size(tc))) == 0;
-    return shape_for(n, vec_ok ? V : 1, t, s);
+    return shape_for(n, access_ok(V, n, tb, tc, B, ldb, C, ldc) ? V : 1, t, s);
 }
 
 // The hybrid row split reads float32 rows of B as two 16-byte vectors per
@@ -197,34 +196,116 @@ int default_slabs(int alg, int k, int n, int b_type) {
     return row_bytes >= min_row ? 2 : 1;
 }
 
+size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
+
+// Workspace of a merge: the boundaries of num_tiles merge-path tiles, and for
+// every CTA (of warps tiles each) the row it carries out, the row it finishes
+// for an earlier CTA, and their partial sums.
 struct MergeLayout {
-    int num_tiles;
+    int num_tiles, ctas;
     size_t off_limits, off_carry_row, off_head_row, off_carry, off_head, total;
 };
 
-size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
-
-MergeLayout merge_layout_items(int m, long long nnz, int n, long long ipt) {
+MergeLayout merge_layout(int m, long long nnz, int n, long long items_per_tile, int warps) {
     MergeLayout L{};
     const long long total = (long long)m + nnz;
-    L.num_tiles = (int)((total + ipt - 1) / ipt);
+    L.num_tiles = (int)((total + items_per_tile - 1) / items_per_tile);
+    L.ctas = (L.num_tiles + warps - 1) / warps;
     size_t off = 0;
     L.off_limits = off;
     off = align256(off + (size_t)(L.num_tiles + 1) * sizeof(int2));
     L.off_carry_row = off;
-    off = align256(off + (size_t)L.num_tiles * 4);
+    off = align256(off + (size_t)L.ctas * 4);
     L.off_head_row = off;
-    off = align256(off + (size_t)L.num_tiles * 4);
+    off = align256(off + (size_t)L.ctas * 4);
     L.off_carry = off;
-    off = align256(off + (size_t)L.num_tiles * n * 4);
+    off = align256(off + (size_t)L.ctas * n * 4);
     L.off_head = off;
-    off = align256(off + (size_t)L.num_tiles * n * 4);
+    off = align256(off + (size_t)L.ctas * n * 4);
     L.total = off;
     return L;
 }
 
-MergeLayout merge_layout(int m, long long nnz, int n, const Shape& s) {
-    return merge_layout_items(m, nnz, n, (long long)(merge_cta_threads(s.W) / s.W) * s.ips);
+// Whether the merge based algorithm runs merge_kernel_narrow (lane groups walk
+// separate shares of a CTA's tile) or merge_kernel (a warp's lanes walk one
+// tile together) for column slabs of shape s.  With W lanes per row the warp
+// adds up 32 / W lane groups' partial sums at every row end, which short rows
+// do not repay: up to 4 lanes of 16 bytes, 8 lanes below a mean of 4 nonzeros
+// per row and unaligned rows of up to 4 columns below 8 run the narrow kernel.
+// Measured on GB300, narrow / the other (us): 300,000 rows of Poisson 8,
+// n = 16, 41 / 51; 400,000 of Poisson 2.5, n = 32, 42 / 46; 700,000 of Poisson
+// 5, n = 32, 94 / 88; 700,000 of Poisson 5, n = 2, 43 / 55.
+bool merge_narrow(int m, long long nnz, const Shape& s) {
+    if (s.vec > 1) return s.W <= 4 || (s.W == 8 && nnz < 4LL * m);
+    return s.W <= 4 && nnz < 8LL * m;
+}
+
+// Lane layout of the merge based kernels where 16-byte accesses are not
+// aligned (base.vec == 1).  merge_kernel then covers up to 128 columns in one
+// pass over A: 32 lanes with up to 4 chunks of one element or, where two
+// elements are aligned, 2 chunks of two (a chunk of a row of B is one request
+// of 128 or 256 consecutive bytes), or one element and as many lanes as needed
+// for up to 32 columns.  Measured on GB300, 250,000 rows of a graph of mean
+// degree 20, n = 47: two passes of 32 columns 0.165 ms, one of two chunks
+// 0.12 ms.
+Shape merge_shape(const Shape& base, int n, int tb, int tc, const void* B, long long ldb, const void* C, long long ldc,
+                  const spmm_tuning_t& t) {
+    if (base.ips > 0 || base.vec > 1) return base;
+    const long long passes = t.lanes_per_row > 0 ? base.slabs : std::max<long long>(t.column_slabs, (n + 127) / 128);
+    const long long want = (n + passes - 1) / passes;  // columns per slab
+    Shape s = base;
+    s.vec = want > 32 && access_ok(2, n, tb, tc, B, ldb, C, ldc) ? 2 : 1;
+    s.W = pow2_ceil((want + s.vec - 1) / s.vec);
+    while (s.vec * s.chunks < 4 && 32LL * s.vec * s.chunks < want) s.chunks <<= 1;
+    const long long cols = (long long)s.W * s.vec * s.chunks;
+    s.slabs = (int)((n + cols - 1) / cols);
+    return s;
+}
+
+// Merge-path items per lane group of merge_kernel_narrow: tiles of kNarrowTile
+// items, or smaller ones that make one or two whole waves of its persistent
+// CTAs (6 per SM) where kNarrowTile would make at most two.  400,000 rows of
+// Poisson 2.5, n = 32: 1.5 waves of 1024 items 47 us, 2 of 768 42 us.
+int narrow_items(long long total, int groups) {
+    const long long wave = 6 * 152;
+    long long items = kNarrowTile;
+    if (total < wave * kNarrowTile * 2) {
+        const long long waves = total < wave * kNarrowTile * 5 / 8 ? 1 : 2;
+        items = std::max<long long>(128, (total + waves * wave - 1) / (waves * wave));
+    }
+    return std::max(4, (int)((items + groups - 1) / groups));
+}
+
+// Merge-path items per tile; sets s->ips, which is not 0 for the narrow kernel
+// only.  The caller's items_per_subwarp counts per lane group of a block of 256
+// threads (128 for up to 8 lanes per row), for the tiles of a whole CTA.  By
+// default a warp of merge_kernel takes about kMergeTile items, so that the
+// tiles make whole waves of the warps that the GPU runs at once (28 or 32 per
+// SM): a wave filled to a tenth costs as much as a full one.  300,000 rows of
+// Poisson 8, n = 128: 1.08 waves of 512 items 190 us, one wave of 555 147 us.
+// Where the partial sums are large (over 8 MiB) no tile is smaller than the full
+// one, so that a workspace of 16 MiB fits whatever it fitted with full tiles.
+constexpr int kMergeTile = 512;
+long long merge_tile(int m, long long nnz, int n, const spmm_tuning_t* t, int sv, Shape* s) {
+    const int groups = (s->W >= 16 ? 256 : 128) / s->W;
+    const int asked = t && t->items_per_subwarp > 0 ? std::min(std::max(t->items_per_subwarp, 4), 4096) : 0;
+    const long long total = (long long)m + nnz;
+    s->ips = 0;
+    if (merge_narrow(m, nnz, *s)) {
+        const bool large = total / kNarrowTile * n * 8 > (8LL << 20);
+        s->ips = asked ? asked : large ? kNarrowTile / groups : narrow_items(total, groups);
+        auto smem = [&]() -> size_t {
+            if (sv == 4) return s->vec == 1 ? merge_smem_vec<float, 1>(*s) : s->vec == 4 ? merge_smem_vec<float, 4>(*s) : merge_smem_vec<float, 8>(*s);
+            return s->vec == 1 ? merge_smem_vec<__half, 1>(*s) : s->vec == 4 ? merge_smem_vec<__half, 4>(*s) : merge_smem_vec<__half, 8>(*s);
+        };
+        while (s->ips > 4 && smem() > kMaxSmem) s->ips = s->ips * 3 / 4;  // until the double-buffered staging fits
+        return (long long)groups * s->ips;
+    }
+    if (asked) return ((long long)groups * asked + kMergeWarps - 1) / kMergeWarps;
+    const long long per_wave = (s->W < 32 ? 28LL : 32LL) * 152, wave = kMergeTile * per_wave;
+    const bool large = total / kMergeTile / kMergeWarps * n * 8 > (8LL << 20);
+    const long long tiles = std::max<long long>(1, (total + (large ? 0 : wave / 2)) / wave) * per_wave;
+    return std::max<long long>(64, (total + tiles - 1) / tiles);
 }
 
 // Hybrid row split (SPMM_ALG_ROW_SPLIT_HYBRID).  A lane group of W lanes
@@ -304,16 +385,6 @@ int sm_count() {
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     return n;
-}
-
-// Shrink the merge tile until the double-buffered staging fits one CTA's
-// shared memory (sv = bytes per value; the float32 bound covers 16-bit vals).
-void clamp_tile(Shape* s, int sv) {
-    auto bytes = [&](const Shape& t) -> size_t {
-        if (sv == 4) return t.vec == 1 ? merge_smem_vec<float, 1>(t) : t.vec == 4 ? merge_smem_vec<float, 4>(t) : merge_smem_vec<float, 8>(t);
-        return t.vec == 1 ? merge_smem_vec<__half, 1>(t) : t.vec == 4 ? merge_smem_vec<__half, 4>(t) : merge_smem_vec<__half, 8>(t);
-    };
-    while (s->ips > 4 && bytes(*s) > kMaxSmem) s->ips = s->ips * 3 / 4;
 }
 
 // Stream-ordered allocations of this library come from the device's default
@@ -531,16 +602,10 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
         return cuda_status(L->rowsplit(ra, shape, s));
     }
 
-    // merge based: partition, compute, fix-up.  SpMM tiles are capped so that
-    // the double-buffered staging fits the shared memory of one CTA.
+    // merge based: partition, compute, fix-up
     const int spmv_t = spmv_items(&t_eff);
-    long long ipt = (long long)kThreads * spmv_t;
-    if (!spmv) {
-        clamp_tile(&shape, dtype_size(vals_type));
-        if (L->merge_smem(shape) > kMaxSmem) return SPMM_ERR_INVALID_VALUE;
-        ipt = (long long)(merge_cta_threads(shape.W) / shape.W) * shape.ips;
-    }
-    const MergeLayout lay = merge_layout_items(m, nnz, n, ipt);
+    const long long ipt = spmv ? (long long)kThreads * spmv_t : merge_tile(m, nnz, n, &t_eff, dtype_size(vals_type), &shape);
+    const MergeLayout lay = merge_layout(m, nnz, n, ipt, spmv || shape.ips > 0 ? 1 : kMergeWarps);
     bool own = false;
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     if (!ws) {
@@ -567,20 +632,21 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
     ma.ldc = ldc;
     ma.limits = reinterpret_cast<const int2*>(ws + lay.off_limits);
     ma.num_tiles = lay.num_tiles;
-    ma.slabs = shape.slabs;
-    ma.ips = shape.ips;
     ma.carry = reinterpret_cast<float*>(ws + lay.off_carry);
     ma.head = reinterpret_cast<float*>(ws + lay.off_head);
     ma.carry_row = reinterpret_cast<int*>(ws + lay.off_carry_row);
     ma.head_row = reinterpret_cast<int*>(ws + lay.off_head_row);
     ma.status = d_status;
+    ma.ips = shape.ips;
     ma.use_tma = ((uintptr_t)row_ptr % 16 == 0) && ((uintptr_t)col_ind % 16 == 0) && ((uintptr_t)vals % 16 == 0);
     ma.wait_ns = kWaitLimitNs;
 
+    if (!spmv) shape = merge_shape(shape, n, b_type, c_type, B, ldb, C, ldc, t_eff);
+    ma.slabs = shape.slabs;
     st = spmm_merge_partition(m, nnz, row_ptr, (int)ipt, lay.num_tiles, reinterpret_cast<int*>(ws + lay.off_limits),
                               stream);
     if (st == SPMM_OK) st = cuda_status(spmv ? L->spmv_merge(ma, spmv_t, s) : L->merge(ma, shape, sm_count(), s));
-    if (st == SPMM_OK && lay.num_tiles > 1) st = cuda_status(L->fixup(ma, s));
+    if (st == SPMM_OK && lay.ctas > 1) st = cuda_status(L->fixup(ma, lay.ctas, s));
     if (own) {
         const cudaError_t e = cudaFreeAsync(ws, s);
         if (st == SPMM_OK && e != cudaSuccess) st = cuda_status(e);
@@ -697,13 +763,13 @@ size_t spmm_csr_workspace_size(int m, int k, int n, long long nnz, int alg, int 
             if (slabs) t.column_slabs = slabs;
             Shape s;
             if (!shape_for(n, vec, &t, &s)) return 0;
-            clamp_tile(&s, 4);
-            const size_t need = merge_layout(m, nnz, n, s).total;
+            const long long items = merge_tile(m, nnz, n, &t, 4, &s);
+            const size_t need = merge_layout(m, nnz, n, items, s.ips > 0 ? 1 : kMergeWarps).total;
             if (need > best) best = need;
         }
     }
     if (n == 1) {  // the SpMV form's tiles
-        const size_t need = merge_layout_items(m, nnz, n, (long long)kThreads * spmv_items(tuning)).total;
+        const size_t need = merge_layout(m, nnz, n, (long long)kThreads * spmv_items(tuning), 1).total;
         if (need > best) best = need;
     }
     return best;

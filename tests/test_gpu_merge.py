@@ -1,0 +1,54 @@
+"""GPU parity of the merge-path compute kernel over its lane layouts: every access width and
+alignment, tile and batch edges, empty rows and rows that cross warps and CTAs.
+
+Small integers make every product and partial sum exact in float32, so the result must equal the
+oracle's whatever the summation order."""
+import numpy as np
+import pytest
+
+import oracle
+from spmm_cases import csr_arrays
+
+pytestmark = pytest.mark.gpu
+
+
+def edge_lengths(rng):
+    """Row lengths at the edges of a batch of 32 nonzeros, runs of empty rows, short rows, and rows that span
+    several warps' tiles and several CTAs."""
+    parts = [np.arange(0, 70), np.zeros(200), np.ones(90), [31, 32, 33, 0, 0, 32, 64, 63, 65, 0], rng.integers(0, 4, 700),
+             [6000], np.zeros(40), rng.integers(0, 40, 300), [0, 1500, 0, 0, 511, 512, 513], np.zeros(3)]
+    return np.concatenate(parts).astype(np.int64)
+
+
+@pytest.mark.parametrize("n", [2, 3, 5, 8, 13, 16, 20, 31, 32, 33, 34, 47, 64, 66, 96, 100, 127, 128, 130, 257])
+@pytest.mark.parametrize("pad", [0, 1, 2, 4])
+def test_layouts_are_bitwise(gpu_lib, n, pad):
+    """pad: ldb - n and ldc - n, which with n decides the aligned access width."""
+    import torch
+
+    rng = np.random.default_rng(100 * n + pad)
+    rp, ci, v = csr_arrays(edge_lengths(rng), 7000, 3, int_vals=True)
+    B = rng.integers(-4, 5, size=(7000, n + pad)).astype(np.float32)
+    ref = oracle.spmm(rp, ci, v, np.ascontiguousarray(B[:, :n])).astype(np.float32)
+    d_rp, d_ci, d_v, d_B = (torch.from_numpy(x).cuda() for x in (rp, ci, v, B))
+    for tuning in (None, dict(items_per_subwarp=4), dict(items_per_subwarp=13, column_slabs=2)):
+        out = torch.full((len(rp) - 1, n + pad), 7.0, device="cuda")
+        gpu_lib.spmm(d_rp, d_ci, d_v, d_B[:, :n], alg="merge", out=out[:, :n], nnz=int(rp[-1]), tuning=tuning)
+        got = out.cpu().numpy()
+        assert np.array_equal(got[:, :n], ref), tuning
+        assert np.all(got[:, n:] == 7.0)  # padding untouched
+
+
+@pytest.mark.parametrize("storage", ["bfloat16", "float16"])
+@pytest.mark.parametrize("n", [4, 7, 8, 24, 33, 40, 64, 100, 128, 136, 256])
+def test_16bit_layouts_are_bitwise(gpu_lib, storage, n):
+    import torch
+
+    rng = np.random.default_rng(n)
+    rp, ci, v = csr_arrays(edge_lengths(rng), 7000, 5, int_vals=True)
+    B = rng.integers(-4, 5, size=(7000, n)).astype(np.float32)
+    dt = getattr(torch, storage)
+    d_rp, d_ci = (torch.from_numpy(x).cuda() for x in (rp, ci))
+    C = gpu_lib.spmm(d_rp, d_ci, torch.from_numpy(v).cuda().to(dt), torch.from_numpy(B).cuda().to(dt), alg="merge",
+                     out_dtype=torch.float32, nnz=int(rp[-1]))
+    assert np.array_equal(C.cpu().numpy(), oracle.spmm(rp, ci, v, B).astype(np.float32))
