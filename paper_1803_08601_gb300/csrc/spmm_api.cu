@@ -177,10 +177,23 @@ bool hybrid_two_vectors(int n, int b_type, long long ldb, long long ldc, const S
     return b_type == SPMM_F32 && s.vec == 4 && n >= 32 && n % 8 == 0 && ldb % 8 == 0 && ldc % 8 == 0;
 }
 
-// Column slabs when B is much larger than L2 and its rows are wide: each pass
-// then gathers half of every row, over a B slab twice as likely to be found in
-// L2 (measured on GB300: merge with 512-byte rows and row split with >= 256-byte
-// rows of a B beyond L2 gain 6-14 %; narrower rows lose).
+// Column slabs: each pass gathers a part of every row, over a B slab that much
+// smaller and so more likely to be found in L2.
+//
+// Row split: slabs of 128 bytes (one request of 8 lanes) once B exceeds the five
+// eighths of L2 that uniform gathers can count on, if they divide a row of 256
+// bytes or more with at most a seventh of the last pass to spare.  A pass costs
+// another read of A and another walk, which rows of B of 128 bytes repay as soon
+// as the gathers miss.  Measured on GB300, one pass (above 2 L2: two) against
+// passes of 128 bytes: bf16 n = 128, 1M rows of 32, 0.99 -> 0.81 ms; float32
+// n = 128, 500,000 of 32, 0.93 -> 0.59; 1M of 16, 0.96 -> 0.90; n = 256, 500,000
+// of 32, 1.86 -> 1.18; n = 64, 500,000 of 32, 0.36 -> 0.29; B of 82 MB, n = 128,
+// 0.209 -> 0.199 ms, of 66 MB 0.188 -> 0.197 ms; n = 100 (four passes for 3.1)
+// 0.264 -> 0.291 ms.
+//
+// Otherwise 2 when B is larger than twice L2 and its rows are wide (merge with
+// 512-byte rows, the hybrid and ragged row splits from 256 bytes gain 6-14 %;
+// narrower rows lose).
 int default_slabs(int alg, int k, int n, int b_type) {
     static std::atomic<int> l2_cache[64];  // 0 until first queried; every thread stores the same value
     int dev = 0;
@@ -191,6 +204,10 @@ int default_slabs(int alg, int k, int n, int b_type) {
         l2_cache[dev].store(l2, std::memory_order_relaxed);
     }
     const long long row_bytes = (long long)n * dtype_size(b_type);
+    const long long pieces = (row_bytes + 127) / 128;
+    if (alg == SPMM_ALG_ROW_SPLIT && row_bytes >= 256 && (long long)k * row_bytes > l2 * 5LL / 8 &&
+        pieces * 128 * 7 <= row_bytes * 8)
+        return (int)std::min<long long>(pieces, 65535);
     if ((long long)k * row_bytes <= 2LL * l2) return 1;
     const long long min_row = alg == SPMM_ALG_MERGE ? 512 : 256;
     return row_bytes >= min_row ? 2 : 1;
