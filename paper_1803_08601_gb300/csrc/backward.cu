@@ -16,6 +16,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <climits>
+
 #include "launch.cuh"
 
 namespace spmm {
@@ -339,98 +341,194 @@ __global__ void __launch_bounds__(kThreads) sddmm_kernel(SddmmArgs a) {
     }
 }
 
-// Wide rows (16 to 256 16-byte vectors): a warp per run of `chunk`
-// consecutive nonzeros.  Its first row comes from a 32-ary warp search of
-// row_ptr; the current row of dC stays in registers (lane l holds vectors
-// l, l + 32, ...) and is reloaded only when the row changes; up to U nonzeros
-// of one row are done together, their rows of B gathered with independent
-// loads (U * CPL vectors in flight per lane), and each dot product is reduced
-// across the warp with xor shuffles in the same order as sddmm_kernel.
-template <typename TD, typename TO, int CPL, int U>
-__global__ void __launch_bounds__(kThreads) sddmm_warp_kernel(SddmmArgs a) {
-    constexpr int VEC = Elem<TD>::kVec;
+// Wide and unaligned rows: a warp per run of `chunk` consecutive nonzeros, 32
+// lanes on one nonzero at a time, E column chunks of VEC elements per lane from
+// column col0 on.  U rows of B are gathered before the first is used, whatever
+// rows of A they belong to; the current row of dC stays in registers and changes
+// at the row ends, which are warp-uniform (redux results, kept in uniform
+// registers), with the next row's already on its way.  The U dot products are
+// reduced together: each exchange halves the products a lane holds, so that U =
+// 8 of them take 9 shuffles and not 40.  With `accumulate` a pass adds to what
+// the passes over the columns before col0 left in out (float32).
+//
+// What bounds it is the gathers of B, as in the forward product.  Measured on
+// GB300 (CUDA events, float32) against the kernel that cut its batches at row
+// ends and reduced each product on its own: 500,000-node graph
+// of mean degree 20, n = 256 (two passes), 0.963 -> 0.907 ms (5.1 TB/s of DRAM
+// traffic), n = 128 0.582 -> 0.432; 250,000 nodes, n = 47, 0.710 -> 0.151;
+// 60,000 rows of Poisson 15, n = 128, 0.072 -> 0.045 ms.
+template <typename TD, int VEC, int E>
+__host__ __device__ constexpr int sddmm_unroll() {
+    constexpr int bytes = VEC * E * (int)sizeof(TD);
+    return bytes <= 16 ? 8 : bytes <= 32 ? 4 : bytes <= 64 ? 2 : 1;
+}
+
+// CTAs of 4 warps per SM: 64 registers, more where a lane holds more than 16
+// columns of the row of dC (and of the next one).
+template <int VEC, int E>
+__host__ __device__ constexpr int sddmm_min_blocks() { return VEC * E <= 16 ? 8 : VEC * E <= 32 ? 4 : 2; }
+
+template <typename TD, typename TO, int VEC, int E>
+__global__ void __launch_bounds__(128, sddmm_min_blocks<VEC, E>()) sddmm_warp_kernel(SddmmArgs a, int col0, int accumulate) {
+    constexpr int U = sddmm_unroll<TD, VEC, E>();
+    constexpr int SS = U >= 4 ? 4 : U;  // columns per shared-memory read
+    __shared__ __align__(16) int s_col[4][32];
     const int lane = threadIdx.x & 31;
-    const long long wid = ((long long)blockIdx.x * kThreads + threadIdx.x) >> 5;
-    const long long p0 = wid * a.chunk;
-    if (p0 >= a.nnz) return;  // whole warps leave together
-    const long long p1 = p0 + a.chunk < a.nnz ? p0 + a.chunk : a.nnz;
-    const TD* __restrict__ dC = static_cast<const TD*>(a.dC);
-    const TD* __restrict__ B = static_cast<const TD*>(a.B);
-    const int nchunks = a.n / VEC;
+    const int warp = uniform(threadIdx.x >> 5);
+    const long long first = ((long long)blockIdx.x * 4 + warp) * a.chunk;
+    if (first >= a.nnz) return;  // whole warps leave together
+    const int p0 = uniform((int)first);
+    const int p1 = uniform((int)(first + a.chunk < a.nnz ? first + a.chunk : a.nnz));
+    int* const w_col = s_col[warp];
+    bool col_ok[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) col_ok[e] = col0 + (e * 32 + lane) * VEC < a.n;
+    const int my_col = col_ok[0] ? col0 + lane * VEC : 0;  // lanes past n read along with column 0 and add nothing
+    const TD* const b_col = static_cast<const TD*>(a.B) + my_col;
+    const TD* const d_col = static_cast<const TD*>(a.dC) + my_col;
+    const unsigned ldb_bytes = (unsigned)(a.ldb * (long long)sizeof(TD));
+
     // first row: the largest r with row_ptr[r] <= p0 (row_ptr[0] = 0 <= p0 always holds)
     int lo = 0, hi = a.m;  // answer in [lo, hi)
     while (hi - lo > 1) {
         const long long span = hi - lo;
         const int x = lo + (int)((span * lane) / 32);
-        const unsigned ball = __ballot_sync(kFullMask, (long long)__ldg(a.row_ptr + x) <= p0);
+        const unsigned ball = __ballot_sync(kFullMask, __ldg(a.row_ptr + x) <= p0);
         const int cnt = __popc(ball);  // a prefix of the lanes, at least lane 0
         const int x_last = lo + (int)((span * (cnt - 1)) / 32);
         hi = cnt < 32 ? lo + (int)((span * cnt) / 32) : hi;
         lo = x_last;
     }
-    int row = lo;
-    int row_end = __ldg(a.row_ptr + row + 1);
-    float y[CPL][VEC];
-    auto load_row = [&]() {
-#pragma unroll
-        for (int c = 0; c < CPL; ++c) {
-            const int j = lane + 32 * c;
-            if (j < nchunks) load_vec<TD, VEC>(dC + (long long)row * a.lddc + (long long)j * VEC, y[c]);
-            else
-#pragma unroll
-                for (int e = 0; e < VEC; ++e) y[c][e] = 0.0f;
+    // row ends from row window on, one per lane; next_row(q) finds the first row that ends after nonzero q
+    int window = uniform(lo);
+    auto load_ends = [&]() { return lane < a.m - window ? __ldg(a.row_ptr + window + 1 + lane) : INT_MAX; };
+    int ends = load_ends();
+    int row = window, rend = 0;
+    auto next_row = [&](int q) {
+        unsigned after = __ballot_sync(kFullMask, ends > q);
+        while (after == 0u) {
+            window += 32;
+            ends = load_ends();
+            after = __ballot_sync(kFullMask, ends > q);
         }
+        row = min(window + __ffs(after) - 1, a.m - 1);
+        rend = __reduce_min_sync(kFullMask, ends > q && ends < p1 ? ends : INT_MAX);  // p1 on: no other row here
     };
-    load_row();
-    for (long long p = p0; p < p1;) {
-        if (p >= row_end) {  // warp-uniform: the next nonzero belongs to a later row
-            do {
-                ++row;
-                row_end = __ldg(a.row_ptr + row + 1);
-            } while (p >= row_end);
-            load_row();
-        }
-        const long long pe = p1 < (long long)row_end ? p1 : (long long)row_end;
-        const int cnt = pe - p < U ? (int)(pe - p) : U;
-        int cols[U];
+    float y[E][VEC];
+    Raw<TD, VEC> y_next[E];
+    auto load_y = [&](int r) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) cols[u] = u < cnt ? __ldg(a.col_ind + p + u) : 0;
-        Raw<TD, VEC> x[U][CPL];
+        for (int e = 0; e < E; ++e)
+            y_next[e] = col_ok[e] ? load_raw<TD, VEC>(d_col + (long long)r * a.lddc + e * 32 * VEC) : zero_raw<TD, VEC>();
+    };
+    auto take_y = [&]() {
 #pragma unroll
-        for (int u = 0; u < U; ++u)
+        for (int e = 0; e < E; ++e) widen_raw<TD, VEC>(y_next[e], y[e]);
+    };
+    next_row(p0);
+    load_y(row);
+    take_y();
+    int y_row = -1;  // the row in y_next
+    if (row + 1 < a.m) load_y(y_row = row + 1);
+
+    int mc = lane < p1 - p0 ? __ldg(a.col_ind + p0 + lane) : 0;
+    for (int base = p0;;) {
+        __syncwarp();
+        w_col[lane] = mc;  // slots past p1: column 0, a row that exists
+        __syncwarp();
+        const int left = p1 - base;
+        if (left > 32) mc = lane < left - 32 ? __ldg(a.col_ind + base + 32 + lane) : 0;
+#pragma unroll 1
+        for (int rd = 0; rd < 32 / U; ++rd) {
+            const int gl = left - rd * U;  // nonzeros from this group on
+            if (gl <= 0) break;
+            const int q0 = base + rd * U;
+            Raw<TD, VEC> x[U][E];
 #pragma unroll
-            for (int c = 0; c < CPL; ++c) {
-                const int j = lane + 32 * c;
-                x[u][c] = (u < cnt && j < nchunks) ? load_raw<TD, VEC>(gather_row(B, (long long)j * VEC, cols[u], a.ldb))
-                                                   : zero_raw<TD, VEC>();
+            for (int u0 = 0; u0 < U; u0 += SS) {
+                int c[SS];
+                lds_words<SS>(w_col + rd * U + u0, c);
+#pragma unroll
+                for (int i = 0; i < SS; ++i)
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        x[u0 + i][e] = e == 0 || col_ok[e] ? load_raw<TD, VEC>(row_at(b_col, c[i], ldb_bytes) + e * 32 * VEC)
+                                                           : zero_raw<TD, VEC>();
             }
-        float part[U];
+            float part[U];
+            auto product = [&](int u) {
+                part[u] = 0.0f;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            part[u] = 0.0f;
+                for (int e = 0; e < E; ++e) {
+                    float t[VEC];
+                    widen_raw<TD, VEC>(x[u][e], t);
 #pragma unroll
-            for (int c = 0; c < CPL; ++c) {
-                float t[VEC];
+                    for (int i = 0; i < VEC; ++i) part[u] = fmaf(t[i], y[e][i], part[u]);
+                }
+            };
 #pragma unroll
-                for (int e = 0; e < VEC; ++e) t[e] = 0.0f;
-                fma_raw<TD, VEC>(t, 1.0f, x[u][c]);
+            for (int u0 = 0; u0 < U; u0 += SS) {
+                if (rend - q0 >= u0 + SS) {  // no row ends in these products
 #pragma unroll
-                for (int e = 0; e < VEC; ++e) part[u] = fmaf(t[e], y[c][e], part[u]);
+                    for (int i = 0; i < SS; ++i) product(u0 + i);
+                    continue;
+                }
+#pragma unroll
+                for (int i = 0; i < SS; ++i) {
+                    while (rend - q0 <= u0 + i) {  // this nonzero belongs to a later row (once at most)
+                        next_row(q0 + u0 + i);
+                        if (row != y_row) load_y(row);
+                        take_y();
+                        y_row = -1;
+                        if (row + 1 < a.m) load_y(y_row = row + 1);
+                    }
+                    product(u0 + i);
+                }
+            }
+            if (!col_ok[0]) {
+#pragma unroll
+                for (int u = 0; u < U; ++u) part[u] = 0.0f;
+            }
+            // lane l ends up with product l / (32 / U)
+            int off = 16;
+#pragma unroll
+            for (int cnt = U; cnt > 1; cnt >>= 1, off >>= 1) {
+                const bool upper = (lane & off) != 0;
+#pragma unroll
+                for (int i = 0; i < cnt / 2; ++i) {
+                    const float send = upper ? part[i] : part[i + cnt / 2], keep = upper ? part[i + cnt / 2] : part[i];
+                    part[i] = keep + __shfl_xor_sync(kFullMask, send, off);
+                }
+            }
+#pragma unroll
+            for (; off > 0; off >>= 1) part[0] += __shfl_xor_sync(kFullMask, part[0], off);
+            const int mine = lane / (32 / U);
+            if (lane % (32 / U) == 0 && mine < gl) {
+                TO* const o = static_cast<TO*>(a.out) + q0 + mine;
+                *o = Elem<TO>::from_f(accumulate ? Elem<TO>::to_f(*o) + part[0] : part[0]);
             }
         }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-            for (int u = 0; u < U; ++u) part[u] += __shfl_xor_sync(kFullMask, part[u], off);
-        if (lane < cnt) {
-            float mine = part[0];
-#pragma unroll
-            for (int u = 1; u < U; ++u)
-                if (lane == u) mine = part[u];
-            static_cast<TO*>(a.out)[p + lane] = Elem<TO>::from_f(mine);
-        }
-        p += cnt;
+        if (left <= 32) break;
+        base += 32;
     }
+}
+
+template <typename TD, typename TO, int VEC, int E>
+cudaError_t sddmm_warp_launch(const SddmmArgs& a0, cudaStream_t st) {
+    SddmmArgs a = a0;
+    // nonzeros per warp: about 256, in whole waves of the 32 warps that an SM runs at once
+    const long long wave = 256LL * 32 * 152, waves = std::max<long long>(1, (a.nnz + wave / 2) / wave);
+    const long long per_warp = (a.nnz + waves * 32 * 152 - 1) / (waves * 32 * 152);
+    a.chunk = (int)std::max<long long>(32, (per_warp + 31) / 32 * 32);
+    const long long blocks = (a.nnz + 4LL * a.chunk - 1) / (4LL * a.chunk);
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    for (int c = 0; c < a.n; c += 32 * VEC * E) {
+        sddmm_warp_kernel<TD, TO, VEC, E><<<(unsigned)blocks, 128, 0, st>>>(a, c, c > 0);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (c > 0) g_launches.fetch_add(1, std::memory_order_relaxed);  // the caller counts one
+    }
+    return cudaSuccess;
 }
 
 template <typename TD, typename TO, int VEC>
@@ -452,25 +550,42 @@ template <typename TD, typename TO>
 int sddmm_run(const SddmmArgs& a0, cudaStream_t st) {
     SddmmArgs a = a0;
     constexpr int V = Elem<TD>::kVec;
-    const bool vec_ok = a.n % V == 0 && a.lddc % V == 0 && a.ldb % V == 0 && ((uintptr_t)a.dC % 16) == 0 &&
-                        ((uintptr_t)a.B % 16) == 0;
+    auto aligned = [&](int v) {
+        return a.n % v == 0 && a.lddc % v == 0 && a.ldb % v == 0 && ((uintptr_t)a.dC % (v * sizeof(TD))) == 0 &&
+               ((uintptr_t)a.B % (v * sizeof(TD))) == 0;
+    };
+    const bool vec_ok = aligned(V);
     const int vec = vec_ok ? V : 1;
     const long long nchunks = ((long long)a.n + vec - 1) / vec;
     int W = 1;
     while (W < nchunks && W < 32) W <<= 1;
-    // a warp per 256 nonzeros, dC rows in registers: faster than the lane groups from 16 vectors per
-    // row (measured on the GCN workload: n = 64 float32 0.58 ms against 0.71; n = 32 0.56 against 0.38)
-    if (vec_ok && nchunks >= 16 && nchunks <= 256) {
-        a.chunk = 256;
-        const long long warps = (a.nnz + a.chunk - 1) / a.chunk;
-        const long long blocks = (warps * 32 + kThreads - 1) / kThreads;
-        if (blocks > 0x7fffffffLL) return SPMM_ERR_LAUNCH;
-        const int cpl = (int)((nchunks + 31) / 32);
-        if (cpl <= 1) sddmm_warp_kernel<TD, TO, 1, 8><<<(unsigned)blocks, kThreads, 0, st>>>(a);
-        else if (cpl <= 2) sddmm_warp_kernel<TD, TO, 2, 4><<<(unsigned)blocks, kThreads, 0, st>>>(a);
-        else if (cpl <= 4) sddmm_warp_kernel<TD, TO, 4, 2><<<(unsigned)blocks, kThreads, 0, st>>>(a);
-        else sddmm_warp_kernel<TD, TO, 8, 1><<<(unsigned)blocks, kThreads, 0, st>>>(a);
-        return launched(cudaGetLastError());
+    // A warp per nonzero, with the narrowest access that covers the row in one pass of 32 lanes, or
+    // the widest aligned one and several passes (float32 results) or column chunks (16-bit results,
+    // which cannot be added up in place).  The lane groups stay for up to 3 columns and, up to 32
+    // aligned ones (or 8), for rows of A of fewer than 4 nonzeros, where the warp changes rows at
+    // every other nonzero: 600,000 rows of 3, n = 32, 119 us against 129; 2M nonzeros of a graph,
+    // n = 32, 80 against 64; 900,000 of Poisson 15, n = 8, 72 against 31.
+    constexpr bool kPasses = sizeof(TO) == 4;
+    const int n = a.n;
+    int w = V;
+    while (w > 1 && !aligned(w)) w >>= 1;
+    const bool by_groups = n < 4 || (n <= 32 && a.nnz < 4LL * a.m && (n <= 8 || vec_ok)) ||
+                        (!kPasses && n > (w == V ? 256 * V : 128));
+    if (!by_groups) {
+        if (n <= 32) return launched(sddmm_warp_launch<TD, TO, 1, 1>(a, st));
+        if (w >= 2 && n <= 64) return launched(sddmm_warp_launch<TD, TO, 2, 1>(a, st));
+        if constexpr (V == 8) {
+            if (w >= 4 && n <= 128) return launched(sddmm_warp_launch<TD, TO, 4, 1>(a, st));
+        }
+        if (w == V && (n <= 32 * V || kPasses)) return launched(sddmm_warp_launch<TD, TO, V, 1>(a, st));
+        if constexpr (!kPasses) {
+            if (w == V && n <= 64 * V) return launched(sddmm_warp_launch<TD, TO, V, 2>(a, st));
+            if (w == V && n <= 128 * V) return launched(sddmm_warp_launch<TD, TO, V, 4>(a, st));
+            if (w == V) return launched(sddmm_warp_launch<TD, TO, V, 8>(a, st));
+        }
+        if (w >= 2) return launched(sddmm_warp_launch<TD, TO, 2, 2>(a, st));
+        if (n <= 64) return launched(sddmm_warp_launch<TD, TO, 1, 2>(a, st));
+        return launched(sddmm_warp_launch<TD, TO, 1, 4>(a, st));
     }
     a.chunk = 128;  // nonzeros per lane group: longer runs amortise the row search (n = 32: 0.38 -> 0.35 ms)
     const long long groups = (a.nnz + a.chunk - 1) / a.chunk;

@@ -189,6 +189,26 @@ __device__ __forceinline__ void fma_raw(float (&acc)[VEC], float a, const Raw<T,
     }
 }
 
+// out[e] = element e of r.
+template <typename T, int VEC>
+__device__ __forceinline__ void widen_raw(const Raw<T, VEC>& r, float (&out)[VEC]) {
+    if constexpr (VEC == 1) {
+        out[0] = Elem<T>::to_f(r.v);
+    } else if constexpr (sizeof(T) == 4) {
+        out[0] = r.v.x;
+        out[1] = r.v.y;
+        if constexpr (VEC == 4) {
+            out[2] = r.v.z;
+            out[3] = r.v.w;
+        }
+        static_assert(VEC <= 4, "one vector");
+    } else {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) out[e] = 0.0f;
+        fma_raw<T, VEC>(out, 1.0f, r);
+    }
+}
+
 // ------------------------------------------------------------------ semirings
 //
 // C = A (+).(x) B (the GraphBLAS matrix product named in Section 1).  Each tag

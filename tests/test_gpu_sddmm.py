@@ -1,0 +1,46 @@
+"""GPU parity of SDDMM over its lane layouts: every access width and alignment, several passes over
+wide rows, row ends anywhere in a group, empty rows and rows that span many warps.
+
+Small integers make every product and partial sum exact in float32, so float32 results must equal
+the oracle's and 16-bit results its rounding."""
+import numpy as np
+import pytest
+
+import oracle
+from spmm_cases import csr_arrays
+from test_gpu_merge import edge_lengths
+
+pytestmark = pytest.mark.gpu
+
+COMBOS = [("float32", "float32"), ("bfloat16", "float32"), ("bfloat16", "bfloat16"), ("float16", "float16")]
+
+
+@pytest.mark.parametrize("n", [1, 3, 4, 8, 16, 31, 32, 33, 47, 64, 66, 96, 100, 127, 128, 129, 130, 192, 256, 260, 512, 640, 1024, 1040])
+@pytest.mark.parametrize("storage,result", COMBOS)
+def test_layouts_are_bitwise(gpu_lib, n, storage, result):
+    import torch
+
+    rng = np.random.default_rng(n)
+    rp, ci, _ = csr_arrays(edge_lengths(rng), 7000, 9)
+    m, dt = len(rp) - 1, getattr(torch, storage)
+    dC = rng.integers(-3, 4, size=(m, n)).astype(np.float32)
+    B = rng.integers(-4, 5, size=(7000, n)).astype(np.float32)
+    d_rp, d_ci, d_dC, d_B = (torch.from_numpy(x).cuda() for x in (rp, ci, dC, B))
+    out = gpu_lib.sddmm(d_rp, d_ci, d_dC.to(dt), d_B.to(dt), out_dtype=getattr(torch, result))
+    ref = torch.from_numpy(oracle.sddmm(rp, ci, dC, B)).to(getattr(torch, result))
+    assert torch.equal(out.cpu(), ref)
+
+
+@pytest.mark.parametrize("n,pad", [(48, 1), (64, 2), (100, 1), (128, 2), (256, 4), (250, 2)])
+def test_strides(gpu_lib, n, pad):
+    """ldb and lddc above n, down to 4- and 8-byte alignment."""
+    import torch
+
+    rng = np.random.default_rng(n + pad)
+    rp, ci, _ = csr_arrays(edge_lengths(rng), 7000, 10)
+    dC = rng.integers(-3, 4, size=(len(rp) - 1, n + pad)).astype(np.float32)
+    B = rng.integers(-4, 5, size=(7000, n + pad)).astype(np.float32)
+    d_rp, d_ci, d_dC, d_B = (torch.from_numpy(x).cuda() for x in (rp, ci, dC, B))
+    out = gpu_lib.sddmm(d_rp, d_ci, d_dC[:, :n], d_B[:, :n])
+    ref = oracle.sddmm(rp, ci, np.ascontiguousarray(dC[:, :n]), np.ascontiguousarray(B[:, :n]))
+    assert np.array_equal(out.cpu().numpy(), ref.astype(np.float32))
