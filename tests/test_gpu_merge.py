@@ -52,3 +52,18 @@ def test_16bit_layouts_are_bitwise(gpu_lib, storage, n):
     C = gpu_lib.spmm(d_rp, d_ci, torch.from_numpy(v).cuda().to(dt), torch.from_numpy(B).cuda().to(dt), alg="merge",
                      out_dtype=torch.float32, nnz=int(rp[-1]))
     assert np.array_equal(C.cpu().numpy(), oracle.spmm(rp, ci, v, B).astype(np.float32))
+
+
+@pytest.mark.parametrize("n", [1, 8, 32, 100])
+def test_auto_gb300_runs_merge_on_small_type1_matrices(gpu_lib, n):
+    """Where the GB300 rule names the hybrid for a skewed matrix of few nonzeros, the call runs merge: the same
+    bits as a forced merge."""
+    import torch
+
+    rng = np.random.default_rng(n)
+    rp, ci, v = csr_arrays(np.concatenate([rng.integers(0, 9, 4000), [3000]]), 5000, 4)
+    d_rp, d_ci, d_v = (torch.from_numpy(x).cuda() for x in (rp, ci, v))
+    B = torch.randn(5000, n, device="cuda")
+    nnz = int(rp[-1])
+    auto = gpu_lib.spmm(d_rp, d_ci, d_v, B, alg="auto_gb300", nnz=nnz)
+    assert torch.equal(auto, gpu_lib.spmm(d_rp, d_ci, d_v, B, alg="merge", nnz=nnz))
