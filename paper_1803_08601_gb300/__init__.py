@@ -173,7 +173,7 @@ def spmm_csr(m, k, n, row_ptr, col_ind, vals, B, ldb, C, ldc, alg, stream) -> in
 
 def spmm_csr_ex(m, k, n, nnz, row_ptr, col_ind, vals, vals_type, B, b_type, ldb, C, c_type, ldc, alg, tuning,
                 workspace, workspace_bytes, d_status, stream) -> int:
-    return load().spmm_csr_ex(m, k, n, nnz, row_ptr, col_ind, vals, vals_type, B, b_type, ldb, C, c_type, ldc, alg,
+    return (_lib or load()).spmm_csr_ex(m, k, n, nnz, row_ptr, col_ind, vals, vals_type, B, b_type, ldb, C, c_type, ldc, alg,
                               _tuning_ptr(tuning), workspace, workspace_bytes, d_status, stream)
 
 
@@ -252,23 +252,32 @@ def _tuning_ptr(t):
         return None
     if isinstance(t, dict):
         t = SpmmTuning(**t)
-    return ctypes.pointer(t)
+    return ctypes.byref(t)
 
 
 # ----------------------------------------------------------------------------- tensor helpers
 
-def _torch():
-    import torch
+_torch_module = None
+_dtype_codes: dict = {}
 
-    return torch
+
+def _torch():
+    global _torch_module
+    if _torch_module is None:
+        import torch
+
+        _dtype_codes.update({torch.float32: F32, torch.bfloat16: BF16, torch.float16: F16})
+        _torch_module = torch
+    return _torch_module
 
 
 def dtype_code(dt) -> int:
-    torch = _torch()
-    m = {torch.float32: F32, torch.bfloat16: BF16, torch.float16: F16}
-    if dt not in m:
+    if _torch_module is None:
+        _torch()
+    code = _dtype_codes.get(dt)
+    if code is None:
         raise TypeError(f"unsupported dtype {dt}")
-    return m[dt]
+    return code
 
 
 def alg_code(alg) -> int:
@@ -281,9 +290,13 @@ def _check(status: int, where: str):
 
 
 def _stream_handle(stream=None) -> int:
+    if stream is not None:
+        return int(stream.cuda_stream)
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return int(s.cuda_stream)
+    if not torch.cuda.is_initialized():
+        return int(torch.cuda.current_stream().cuda_stream)
+    # the handle alone: a Stream object of the current stream costs about 3 us per call
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _require_cuda(*ts):
@@ -309,13 +322,14 @@ def spmm(row_ptr, col_ind, vals, B, alg="auto", out=None, out_dtype=None, nnz=No
         raise ValueError("B must be a row-major 2-D tensor")
     m = row_ptr.numel() - 1
     k, n = B.shape
+    b_dtype = B.dtype
     if out is None:
-        out = torch.empty((m, n), dtype=out_dtype or B.dtype, device=B.device)
-    if out.dim() != 2 or out.shape != (m, n) or out.stride(1) != 1:
+        out = torch.empty((m, n), dtype=out_dtype or b_dtype, device=B.device)
+    elif out.dim() != 2 or out.shape != (m, n) or out.stride(1) != 1:
         raise ValueError("out must be a row-major [m, n] tensor")
     ws_ptr, ws_bytes = (workspace.data_ptr(), workspace.numel() * workspace.element_size()) if workspace is not None else (None, 0)
     st = spmm_csr_ex(m, k, n, -1 if nnz is None else int(nnz), row_ptr.data_ptr(), col_ind.data_ptr(),
-                     vals.data_ptr(), dtype_code(vals.dtype), B.data_ptr(), dtype_code(B.dtype), B.stride(0),
+                     vals.data_ptr(), dtype_code(vals.dtype), B.data_ptr(), dtype_code(b_dtype), B.stride(0),
                      out.data_ptr(), dtype_code(out.dtype), out.stride(0), alg_code(alg), tuning, ws_ptr, ws_bytes,
                      status.data_ptr() if status is not None else None, _stream_handle(stream))
     _check(st, "spmm_csr_ex")

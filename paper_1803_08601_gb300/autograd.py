@@ -10,7 +10,7 @@ from __future__ import annotations
 
 import torch
 
-from . import ALG_AUTO_GB300, csr_transpose, gather_values, max_row_length, sddmm, spmm
+from . import ALG_AUTO_GB300, SpmmTuning, csr_transpose, gather_values, max_row_length, sddmm, spmm
 
 
 class CSRMatrix:
@@ -23,6 +23,7 @@ class CSRMatrix:
         self.nnz = int(col_ind.numel())
         self._max_row = None
         self._t = None
+        self._t_queued = None
 
     @property
     def max_row(self) -> int:
@@ -30,16 +31,33 @@ class CSRMatrix:
             self._max_row = max_row_length(self.row_ptr)
         return self._max_row
 
+    def queue_transpose(self):
+        """Queue the construction of A^T on the current stream, if it is not there yet, without waiting for it.
+        Work queued on the stream before transpose_pattern() is called overlaps that call's wait."""
+        if self._t is None and self._t_queued is None:
+            parts = csr_transpose(self.row_ptr, self.col_ind, self.k)
+            probe = torch.cuda.Stream()
+            probe.wait_stream(torch.cuda.current_stream())
+            self._t_queued = (*parts, probe)
+
     def transpose_pattern(self):
         """(row_ptr_t, col_ind_t, perm, max_row_t) of A^T, built on first use."""
         if self._t is None:
-            rpt, cit, perm = csr_transpose(self.row_ptr, self.col_ind, self.k)
-            self._t = (rpt, cit, perm, max_row_length(rpt))
+            self.queue_transpose()
+            rpt, cit, perm, probe = self._t_queued
+            # the longest row is read on a stream of its own, which waits for the transpose only; the call
+            # returns once that stream is done, so the parts are complete for every stream from here on
+            self._t = (rpt, cit, perm, max_row_length(rpt, stream=probe))
+            self._t_queued = None
         return self._t
 
     def spmm(self, vals, B, alg=ALG_AUTO_GB300, **kw):
-        tuning = dict(kw.pop("tuning", None) or {})
-        tuning.setdefault("max_row_len", self.max_row)
+        given = kw.pop("tuning", None)
+        if given:
+            tuning = dict(given)
+            tuning.setdefault("max_row_len", self.max_row)
+        else:
+            tuning = SpmmTuning(max_row_len=self.max_row)
         return spmm(self.row_ptr, self.col_ind, vals, B, alg=alg, nnz=self.nnz, tuning=tuning, **kw)
 
     def spmm_t(self, vals, dC, alg=ALG_AUTO_GB300):
@@ -62,6 +80,8 @@ class SpMMFunction(torch.autograd.Function):
         A = ctx.A
         dC = dC.contiguous()
         dvals = dB = None
+        if ctx.needs_input_grad[2]:
+            A.queue_transpose()  # the SDDMM then runs while the host waits for the transpose's longest row
         if ctx.needs_input_grad[1]:
             dvals = sddmm(A.row_ptr, A.col_ind, dC, B.contiguous(), out_dtype=vals.dtype)
         if ctx.needs_input_grad[2]:
