@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "../../include/spmm.h"
 
 namespace spmm {
@@ -208,6 +210,27 @@ __device__ __forceinline__ void widen_raw(const Raw<T, VEC>& r, float (&out)[VEC
         fma_raw<T, VEC>(out, 1.0f, r);
     }
 }
+
+template <int N> struct IntVec;
+template <> struct IntVec<1> { using type = int; };
+template <> struct IntVec<2> { using type = int2; };
+template <> struct IntVec<4> { using type = int4; };
+
+// N consecutive words of shared memory (N * 4 bytes aligned).
+template <int N, typename T>
+__device__ __forceinline__ void lds_words(const T* p, T (&out)[N]) {
+    using V = typename IntVec<N>::type;
+    const V v = *reinterpret_cast<const V*>(p);
+    const int* w = reinterpret_cast<const int*>(&v);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        if constexpr (std::is_same<T, float>::value) out[i] = __int_as_float(w[i]);
+        else out[i] = w[i];
+    }
+}
+
+// A value that every lane holds, moved to a uniform register.
+__device__ __forceinline__ int uniform(int x) { return __reduce_max_sync(kFullMask, x); }
 
 // ------------------------------------------------------------------ semirings
 //

@@ -113,6 +113,88 @@ __global__ void __launch_bounds__(kThreads) rowsplit_kernel(RowSplitArgs a) {
     rowsplit_row<TV, TB, TC, VEC, W, SR>(a, row, blockIdx.y);
 }
 
+// Rows of B and C without 16-byte alignment, more than 32 columns: a warp per
+// row, E column chunks of VEC elements per lane (VEC = 1, or 2 where two
+// elements are aligned), so that up to 128 columns take one pass over A where
+// one element per lane takes one per 32 columns.  The row's (column, value)
+// pairs come a batch of 32 ahead, one per lane, and are handed out four at a
+// time through a warp-private slot of shared memory.  Measured on GB300 against
+// those passes (us): 300,000 rows of Poisson 8, n = 50 152 -> 111, n = 101 315 ->
+// 158; bf16 n = 100 422 -> 102; 200,000 rows of 32, n = 50 176 -> 108.
+template <typename TV, typename TB, typename TC, int VEC, int E, typename SR = PlusTimes>
+__global__ void __launch_bounds__(kThreads) rowsplit_chunks_kernel(RowSplitArgs a) {
+    constexpr int U = VEC * E >= 4 ? 4 : 8;  // nonzeros in flight
+    __shared__ __align__(16) int s_col[kThreads / 32][32];
+    __shared__ __align__(16) float s_val[kThreads / 32][32];
+    const int lane = threadIdx.x & 31;
+    const int warp = uniform(threadIdx.x >> 5);
+    const long long row = (long long)blockIdx.x * (kThreads / 32) + warp;
+    if (row >= a.m) return;  // whole warp
+    const int col0 = (int)blockIdx.y * (32 * VEC * E) + lane * VEC;
+    bool col_ok[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) col_ok[e] = col0 + e * 32 * VEC < a.n;
+    const TB* const b_col = static_cast<const TB*>(a.B) + col0;
+    const unsigned ldb_bytes = (unsigned)(a.ldb * (long long)sizeof(TB));
+    const TV* __restrict__ vals = static_cast<const TV*>(a.vals);
+    const int rs = uniform(__ldg(a.row_ptr + row)), re = uniform(__ldg(a.row_ptr + row + 1));
+    float acc[E][VEC];
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+#pragma unroll
+        for (int i = 0; i < VEC; ++i) acc[e][i] = SR::identity();
+    int mc = 0;
+    float mv = 0.0f;
+    auto fetch = [&](int base) {
+        if (lane < re - base) {
+            mc = __ldg(a.col_ind + base + lane);
+            mv = load_f(vals + base + lane);
+        }
+    };
+    if (rs < re) fetch(rs);
+    for (int base = rs; base < re;) {
+        __syncwarp();
+        s_col[warp][lane] = mc;
+        s_val[warp][lane] = mv;
+        __syncwarp();
+        const int left = re - base;
+        if (left > 32) fetch(base + 32);
+#pragma unroll 1
+        for (int g = 0; g < 32 / U; ++g) {
+            const int cnt = left - g * U;  // nonzeros from this group on
+            if (cnt <= 0) break;
+            Raw<TB, VEC> bv[U][E];
+            float vv[U];
+#pragma unroll
+            for (int u0 = 0; u0 < U; u0 += 4) {
+                int c[4];
+                float v[4];
+                lds_words<4>(s_col[warp] + g * U + u0, c);
+                lds_words<4>(s_val[warp] + g * U + u0, v);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    vv[u0 + i] = v[i];
+#pragma unroll
+                    for (int e = 0; e < E; ++e)
+                        bv[u0 + i][e] = u0 + i < cnt && col_ok[e]
+                                            ? load_raw<TB, VEC>(row_at(b_col, c[i], ldb_bytes) + e * 32 * VEC)
+                                            : zero_raw<TB, VEC>();
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (u < cnt)
+#pragma unroll
+                    for (int e = 0; e < E; ++e) accum_raw<SR, TB, VEC>(acc[e], vv[u], bv[u][e]);
+        }
+        if (left <= 32) break;
+        base += 32;
+    }
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (col_ok[e]) store_vec<TC, VEC>(static_cast<TC*>(a.C) + row * a.ldc + col0 + e * 32 * VEC, acc[e]);
+}
+
 // ============================================================================ merge path
 //
 // Algorithm II (Section 4.2, Algorithm 1).  The path that merges the row end

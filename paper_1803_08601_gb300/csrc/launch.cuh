@@ -82,9 +82,26 @@ cudaError_t rowsplit_launch_vec(const RowSplitArgs& a, const Shape& s, cudaStrea
     }
 }
 
+template <typename TV, typename TB, typename TC, int VEC, int E, typename SR>
+cudaError_t rowsplit_chunks_launch(const RowSplitArgs& a, const Shape& s, cudaStream_t st) {
+    const long long gx = ((long long)a.m + kThreads / 32 - 1) / (kThreads / 32);
+    if (gx > 0x7fffffffLL || s.slabs > 65535) return cudaErrorInvalidConfiguration;
+    rowsplit_chunks_kernel<TV, TB, TC, VEC, E, SR><<<dim3((unsigned)gx, (unsigned)s.slabs), kThreads, 0, st>>>(a);
+    const cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
+    return e;
+}
+
 template <typename TV, typename TB, typename TC, typename SR>
 cudaError_t rowsplit_launch(const RowSplitArgs& a, const Shape& s, cudaStream_t st) {
     constexpr int V = Elem<TB>::kVec;
+    if (s.W == 32 && s.vec <= 2 && s.vec * s.chunks > 1) {
+        if (s.vec == 2)
+            return s.chunks == 2 ? rowsplit_chunks_launch<TV, TB, TC, 2, 2, SR>(a, s, st)
+                                 : rowsplit_chunks_launch<TV, TB, TC, 2, 1, SR>(a, s, st);
+        return s.chunks == 4 ? rowsplit_chunks_launch<TV, TB, TC, 1, 4, SR>(a, s, st)
+                             : rowsplit_chunks_launch<TV, TB, TC, 1, 2, SR>(a, s, st);
+    }
     return s.vec == 1 ? rowsplit_launch_vec<TV, TB, TC, 1, SR>(a, s, st) : rowsplit_launch_vec<TV, TB, TC, V, SR>(a, s, st);
 }
 
@@ -236,7 +253,7 @@ cudaError_t merge_launch_one(const MergeArgs& a, const Shape& s, cudaStream_t st
     return e;
 }
 
-// The shapes merge_shape (spmm_api.cu) picks: 16-byte accesses, or narrower
+// The shapes unaligned_shape (spmm_api.cu) picks: 16-byte accesses, or narrower
 // ones, from 33 columns on with 32 lanes and up to 4 chunks.
 template <typename TV, typename TB, typename TC, typename SR>
 cudaError_t merge_launch(const MergeArgs& a, const Shape& s, int grid_cap, cudaStream_t st) {

@@ -3,7 +3,6 @@
 #pragma once
 
 #include <climits>
-#include <type_traits>
 
 #include "kernels.cuh"
 
@@ -28,27 +27,6 @@ __host__ __device__ constexpr int merge_min_blocks() {
     constexpr int bytes = VEC * E * (int)sizeof(TB) * merge_unroll<TB, VEC, E, W>();
     return bytes > 64 ? (W < 32 ? 7 : 8) : (VEC == 2 && W == 32) || W < 32 ? 10 : 8;
 }
-
-template <int N> struct IntVec;
-template <> struct IntVec<1> { using type = int; };
-template <> struct IntVec<2> { using type = int2; };
-template <> struct IntVec<4> { using type = int4; };
-
-// N consecutive words of shared memory (N * 4 bytes aligned).
-template <int N, typename T>
-__device__ __forceinline__ void lds_words(const T* p, T (&out)[N]) {
-    using V = typename IntVec<N>::type;
-    const V v = *reinterpret_cast<const V*>(p);
-    const int* w = reinterpret_cast<const int*>(&v);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-        if constexpr (std::is_same<T, float>::value) out[i] = __int_as_float(w[i]);
-        else out[i] = w[i];
-    }
-}
-
-// A value that every lane holds, moved to a uniform register.
-__device__ __forceinline__ int uniform(int x) { return __reduce_max_sync(kFullMask, x); }
 
 // Phase 2 of Algorithm 1.  A warp walks its tile (rows [r0, r1) that end in
 // it, nonzeros [z0, z1)) in order, all lanes on the same row: W lanes hold the

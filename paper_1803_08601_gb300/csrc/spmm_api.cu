@@ -278,18 +278,17 @@ bool merge_narrow(int m, long long nnz, const Shape& s) {
     return s.W <= 4 && nnz < 8LL * m;
 }
 
-// Lane layout of the merge based kernels where 16-byte accesses are not
-// aligned (base.vec == 1).  merge_kernel then covers up to 128 columns in one
-// pass over A: 32 lanes with up to 4 chunks of one element or, where two
-// elements are aligned, 2 chunks of two (a chunk of a row of B is one request
-// of 128 or 256 consecutive bytes), or one element and as many lanes as needed
-// for up to 32 columns.  Measured on GB300, 250,000 rows of a graph of mean
-// degree 20, n = 47: two passes of 32 columns 0.165 ms, one of two chunks
+// Lane layout where 16-byte accesses are not aligned (base.vec == 1): up to 128
+// columns in one pass over A, as many lanes as needed for up to 32 columns, else
+// 32 lanes with up to 4 chunks of one element or, where two elements are
+// aligned, 2 chunks of two (a chunk of a row of B is one request of 128 or 256
+// consecutive bytes).  Measured on GB300, merge on 250,000 rows of a graph of
+// mean degree 20, n = 47: two passes of 32 columns 0.165 ms, one of two chunks
 // 0.12 ms.
-Shape merge_shape(const Shape& base, int n, int tb, int tc, const void* B, long long ldb, const void* C, long long ldc,
-                  const spmm_tuning_t& t) {
-    if (base.ips > 0 || base.vec > 1) return base;
-    const long long passes = t.lanes_per_row > 0 ? base.slabs : std::max<long long>(t.column_slabs, (n + 127) / 128);
+Shape unaligned_shape(const Shape& base, int n, int tb, int tc, const void* B, long long ldb, const void* C,
+                      long long ldc, const spmm_tuning_t* t) {
+    const long long asked = t ? t->column_slabs : 0;  // the default slabs are for aligned rows
+    const long long passes = t && t->lanes_per_row > 0 ? base.slabs : std::max<long long>(asked, (n + 127) / 128);
     const long long want = (n + passes - 1) / passes;  // columns per slab
     Shape s = base;
     s.vec = want > 32 && access_ok(2, n, tb, tc, B, ldb, C, ldc) ? 2 : 1;
@@ -637,6 +636,7 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
         if (spmv)
             return cuda_status(
                 L->spmv_rowsplit(ra, t_eff.lanes_per_row > 0 ? t_eff.lanes_per_row : spmv_lanes(m, nnz), s));
+        if (shape.vec == 1) shape = unaligned_shape(shape, n, b_type, c_type, B, ldb, C, ldc, tuning);
         return cuda_status(L->rowsplit(ra, shape, s));
     }
 
@@ -679,7 +679,8 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
     ma.use_tma = ((uintptr_t)row_ptr % 16 == 0) && ((uintptr_t)col_ind % 16 == 0) && ((uintptr_t)vals % 16 == 0);
     ma.wait_ns = kWaitLimitNs;
 
-    if (!spmv) shape = merge_shape(shape, n, b_type, c_type, B, ldb, C, ldc, t_eff);
+    if (!spmv && shape.vec == 1 && shape.ips == 0)
+        shape = unaligned_shape(shape, n, b_type, c_type, B, ldb, C, ldc, tuning);
     ma.slabs = shape.slabs;
     st = spmm_merge_partition(m, nnz, row_ptr, (int)ipt, lay.num_tiles, reinterpret_cast<int*>(ws + lay.off_limits),
                               stream);
