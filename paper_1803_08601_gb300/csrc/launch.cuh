@@ -43,6 +43,7 @@ struct Launchers {
     SpmvMergeFn spmv_merge;        // n = 1, tiles of kThreads * items_per_thread items (4, 8 or 16)
     TiledFn tiled;                 // A/B tiling; 16-byte vectors only (shape.vec > 1)
     RowSplitHybridFn rowsplit_hybrid;  // row pass + segment pass of the hybrid row split
+    bool plus_times;                   // the ordinary product, not another semiring
 };
 
 // defined in inst_*.cu
@@ -411,7 +412,7 @@ template <typename TV, typename TB, typename TC, typename SR = PlusTimes>
 Launchers make_launchers() {
     return Launchers{&rowsplit_launch<TV, TB, TC, SR>, &merge_launch<TV, TB, TC, SR>, &fixup_launch<TC, SR>,
                      &spmv_rowsplit_launch<TV, TB, TC, SR>, &spmv_merge_launch<TV, TB, TC, SR>,
-                     &tiled_launch<TV, TB, TC, SR>, &hybrid_launch<TV, TB, TC, SR>};
+                     &tiled_launch<TV, TB, TC, SR>, &hybrid_launch<TV, TB, TC, SR>, std::is_same<SR, PlusTimes>::value};
 }
 
 }  // namespace spmm

@@ -201,21 +201,22 @@ bool hybrid_two_vectors(int n, int b_type, long long ldb, long long ldc, const S
 // Column slabs: each pass gathers a part of every row, over a B slab that much
 // smaller and so more likely to be found in L2.
 //
-// Row split: slabs of 128 bytes (one request of 8 lanes) once B exceeds the five
-// eighths of L2 that uniform gathers can count on, if they divide a row of 256
-// bytes or more with at most a seventh of the last pass to spare.  A pass costs
-// another read of A and another walk, which rows of B of 128 bytes repay as soon
-// as the gathers miss.  Measured on GB300, one pass (above 2 L2: two) against
-// passes of 128 bytes: bf16 n = 128, 1M rows of 32, 0.99 -> 0.81 ms; float32
-// n = 128, 500,000 of 32, 0.93 -> 0.59; 1M of 16, 0.96 -> 0.90; n = 256, 500,000
-// of 32, 1.86 -> 1.18; n = 64, 500,000 of 32, 0.36 -> 0.29; B of 82 MB, n = 128,
-// 0.209 -> 0.199 ms, of 66 MB 0.188 -> 0.197 ms; n = 100 (four passes for 3.1)
-// 0.264 -> 0.291 ms.
+// Row split: a pass covers 512 bytes of a row (32 lanes).  Where half of L2 does
+// not hold that much of B, slabs of 256 or 128 bytes do (128 if neither does),
+// for rows of 256 bytes or more (512 for the semirings, whose walk costs more)
+// that leave at most a seventh of the last pass to spare.  A pass costs another
+// read of A and another walk, which is repaid as soon as the gathers miss.
+// Measured on GB300, one pass (above 2 L2: two) against these: bf16 n = 128, 1M
+// rows of 32, 0.99 -> 0.81 ms; float32 n = 128, 500,000 of 32, 0.93 -> 0.59; 1M
+// of 16, 0.96 -> 0.90; n = 256, 500,000 of 32, 1.86 -> 1.18; n = 64, 500,000 of
+// 32, 0.36 -> 0.29; B of 82 MB, n = 128, 0.209 -> 0.192 ms.  Where 512 bytes fit,
+// 128 cost (n = 256, k = 85,000: 0.57 -> 0.66 ms), and so do four passes for the
+// 3.1 of n = 100 (0.264 -> 0.291 ms).
 //
 // Otherwise 2 when B is larger than twice L2 and its rows are wide (merge with
 // 512-byte rows, the hybrid and ragged row splits from 256 bytes gain 6-14 %;
 // narrower rows lose).
-int default_slabs(int alg, int k, int n, int b_type) {
+int default_slabs(int alg, int k, int n, int b_type, bool plus_times) {
     static std::atomic<int> l2_cache[64];  // 0 until first queried; every thread stores the same value
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
@@ -225,10 +226,14 @@ int default_slabs(int alg, int k, int n, int b_type) {
         l2_cache[dev].store(l2, std::memory_order_relaxed);
     }
     const long long row_bytes = (long long)n * dtype_size(b_type);
-    const long long pieces = (row_bytes + 127) / 128;
-    if (alg == SPMM_ALG_ROW_SPLIT && row_bytes >= 256 && (long long)k * row_bytes > l2 * 5LL / 8 &&
-        pieces * 128 * 7 <= row_bytes * 8)
-        return (int)std::min<long long>(pieces, 65535);
+    if (alg == SPMM_ALG_ROW_SPLIT && row_bytes >= (plus_times ? 256 : 512) &&
+        (long long)k * std::min(row_bytes, 512LL) > l2 / 2) {
+        const long long width = (long long)k * 256 <= l2 / 2 ? 256 : 128;
+        for (long long w = width; w >= 128; w /= 2) {
+            const long long pieces = (row_bytes + w - 1) / w;
+            if (pieces * w * 7 <= row_bytes * 8) return (int)std::min<long long>(pieces, 65535);
+        }
+    }
     if ((long long)k * row_bytes <= 2LL * l2) return 1;
     const long long min_row = alg == SPMM_ALG_MERGE ? 512 : 256;
     return row_bytes >= min_row ? 2 : 1;
@@ -584,7 +589,7 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
     if (alg == SPMM_ALG_AUTO_GB300) alg = route_gb300(m, nnz, lmax, n, b_type);
     const int a = resolve_alg(alg, m, nnz, tuning);
     spmm_tuning_t t_eff = tuning ? *tuning : spmm_tuning_t{};
-    if (t_eff.column_slabs <= 0 && t_eff.lanes_per_row <= 0) t_eff.column_slabs = default_slabs(a, k, n, b_type);
+    if (t_eff.column_slabs <= 0 && t_eff.lanes_per_row <= 0) t_eff.column_slabs = default_slabs(a, k, n, b_type, L->plus_times);
     if (!choose_shape(n, b_type, c_type, B, ldb, C, ldc, &t_eff, &shape)) return SPMM_ERR_INVALID_VALUE;
     if (a == SPMM_ALG_ROW_SPLIT_HYBRID && hybrid_two_vectors(n, b_type, ldb, ldc, shape) && !shape_for(n, 8, &t_eff, &shape))
         return SPMM_ERR_INVALID_VALUE;
@@ -760,7 +765,7 @@ double spmm_tiled_reuse(int m, int k, long long nnz, int n, int b_type) {
 
 int spmm_default_column_slabs(int alg, int k, int n, int b_type) {
     if (k < 0 || n < 0 || dtype_size(b_type) == 0) return 1;
-    return spmm::default_slabs(alg, k, n, b_type);
+    return spmm::default_slabs(alg, k, n, b_type, true);
 }
 
 int spmm_csr_max_row_length(int m, const int* row_ptr, long long* max_row_len, void* stream) {

@@ -1,4 +1,4 @@
-"""The row split's default column slabs: 128 bytes of a row of B each once B outgrows L2.  Slabs do not
+"""The row split's default column slabs, once B outgrows L2.  Slabs do not
 change the order of any sum, so the result equals the one-slab result bit for bit."""
 import numpy as np
 import pytest
@@ -7,12 +7,15 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("storage,k,n,slabs", [
-    ("float32", 200_000, 128, 4), ("float32", 130_000, 192, 6), ("float32", 300_000, 96, 3), ("float32", 300_000, 127, 4),
+    ("float32", 200_000, 128, 2),   # 256 bytes per row fit half of L2
+    ("float32", 400_000, 128, 4), ("float32", 140_000, 192, 3), ("float32", 300_000, 192, 6), ("float32", 300_000, 96, 3),
+    ("float32", 300_000, 127, 4),
     ("float32", 300_000, 100, 1),   # four slabs would cover 128 columns
     ("float32", 700_000, 100, 2),   # B above twice the L2: two slabs as for ragged rows
-    ("float32", 100_000, 128, 1),   # B below 5/8 of L2
+    ("float32", 100_000, 128, 1),   # 512 bytes per row fit half of L2
+    ("float32", 100_000, 256, 1),   # a pass covers 512 bytes of the 1024
     ("float32", 900_000, 32, 1),    # rows of 128 bytes
-    ("bfloat16", 400_000, 128, 2), ("bfloat16", 200_000, 256, 4), ("float16", 300_000, 192, 3), ("float16", 300_000, 136, 1)])
+    ("bfloat16", 600_000, 128, 2), ("bfloat16", 400_000, 256, 4), ("float16", 400_000, 192, 3), ("float16", 400_000, 136, 1)])
 def test_default_slabs_do_not_change_a_bit(gpu_lib, storage, k, n, slabs):
     import torch
 
