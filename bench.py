@@ -155,12 +155,22 @@ def subproblem(rows, row_ptr, col_ind, vals, B):
 
 
 GATHER_JSON = os.path.join(ROOT, "profiles", "gather_ceiling_sweep.jsonl")
-TRAFFIC_SOURCES = ["paper_1803_08601_gb300/csrc/kernels.cuh", "paper_1803_08601_gb300/csrc/common.cuh"]
+TRAFFIC_SOURCES = ["paper_1803_08601_gb300/csrc/merge.cuh", "paper_1803_08601_gb300/csrc/kernels.cuh",
+                   "paper_1803_08601_gb300/csrc/common.cuh"]
 TRAFFIC_JSON = os.path.join(ROOT, "profiles", "merge_kernel_power_law_1M_dram.json")
 TRAFFIC_COMMAND = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,lts__t_sector_hit_rate.pct,"
                    "gpu__time_duration.sum --print-units base --clock-control none -k regex:merge_kernel -s 12 -c 4 "
                    "--csv --log-file <CSV> python bench.py --alg merge --steps 1 --warmup 3 --no-extras --forms= "
                    "--no-clocks")
+
+
+def auto_gb300_runs(pkg, pick, nnz, max_row, n):
+    """The family a float32 SPMM_ALG_AUTO_GB300 call runs when the selector's rule names `pick` (include/spmm.h)."""
+    if pick != pkg.ALG_ROW_SPLIT_HYBRID:
+        return pick
+    type1 = max_row > 1024 and max_row * 8192 >= nnz
+    ahead = n > 1 and n % 4 == 0 and ((n <= 16 and nnz >= 8 << 20) if type1 else (n <= 64 and nnz >= 1_500_000))
+    return pick if ahead else pkg.ALG_MERGE
 
 
 def sources_sha256(paths):
@@ -459,7 +469,8 @@ def main():
     max_row = pkg.max_row_length(d_rp)  # measured once; passed to the GB300 selector as a hint
     paper_pick = {n: pkg.spmm_select_alg(m, nnz, 0.0) for n in ns}
     gb300_pick = {n: pkg.spmm_select_alg_gb300(m, nnz, max_row, n, pkg.F32) for n in ns}
-    alg_of = {n: {"auto": paper_pick[n], "auto_gb300": gb300_pick[n]}.get(args.alg, pkg.alg_code(args.alg)) for n in ns}
+    gb300_runs = {n: auto_gb300_runs(pkg, gb300_pick[n], nnz, max_row, n) for n in ns}
+    alg_of = {n: {"auto": paper_pick[n], "auto_gb300": gb300_runs[n]}.get(args.alg, pkg.alg_code(args.alg)) for n in ns}
     tuning_ws = json.loads(args.tuning) if args.tuning else None
     ws_bytes = max(pkg.workspace_size(m, k, n, nnz, al, tuning=tuning_ws)
                    for n in ns for al in (pkg.ALG_MERGE, pkg.ALG_ROW_SPLIT_HYBRID))

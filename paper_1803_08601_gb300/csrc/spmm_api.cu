@@ -210,7 +210,7 @@ bool hybrid_two_vectors(int n, int b_type, long long ldb, long long ldc, const S
 // rows of 32, 0.99 -> 0.81 ms; float32 n = 128, 500,000 of 32, 0.93 -> 0.59; 1M
 // of 16, 0.96 -> 0.90; n = 256, 500,000 of 32, 1.86 -> 1.18; n = 64, 500,000 of
 // 32, 0.36 -> 0.29; B of 82 MB, n = 128, 0.209 -> 0.192 ms.  Where 512 bytes fit,
-// 128 cost (n = 256, k = 85,000: 0.57 -> 0.66 ms), and so do four passes for the
+// 128 cost (n = 256, 200,000 rows of 37, k = 85,000: 0.37 -> 0.41 ms), and so do four passes for the
 // 3.1 of n = 100 (0.264 -> 0.291 ms).
 //
 // Otherwise 2 when B is larger than twice L2 and its rows are wide (merge with
@@ -334,7 +334,7 @@ long long merge_tile(int m, long long nnz, int n, const spmm_tuning_t* t, int sv
     const long long total = (long long)m + nnz;
     s->ips = 0;
     if (merge_narrow(m, nnz, *s)) {
-        const bool large = total / kNarrowTile * n * 8 > (8LL << 20);
+        const bool large = std::max(total / kNarrowTile, 2LL * 6 * 152) * n * 8 > (8LL << 20);
         s->ips = asked ? asked : large ? kNarrowTile / groups : narrow_items(total, groups);
         auto smem = [&]() -> size_t {
             if (sv == 4) return s->vec == 1 ? merge_smem_vec<float, 1>(*s) : s->vec == 4 ? merge_smem_vec<float, 4>(*s) : merge_smem_vec<float, 8>(*s);
@@ -345,15 +345,19 @@ long long merge_tile(int m, long long nnz, int n, const spmm_tuning_t* t, int sv
     }
     if (asked) return ((long long)groups * asked + kMergeWarps - 1) / kMergeWarps;
     const long long per_wave = (s->W < 32 ? 28LL : 32LL) * 152, wave = kMergeTile * per_wave;
-    const bool large = total / kMergeTile / kMergeWarps * n * 8 > (8LL << 20);
-    const long long tiles = std::max<long long>(1, (total + (large ? 0 : wave / 2)) / wave) * per_wave;
-    return std::max<long long>(64, (total + tiles - 1) / tiles);
+    long long tiles = std::max<long long>(1, (total + wave / 2) / wave) * per_wave;
+    if (tiles / kMergeWarps * n * 8 > (8LL << 20)) tiles = total / wave * per_wave;  // large: rounded down
+    return tiles == 0 ? kMergeTile : std::max<long long>(64, (total + tiles - 1) / tiles);
 }
 
 // Hybrid row split (SPMM_ALG_ROW_SPLIT_HYBRID).  A lane group of W lanes
 // takes BS = max(W, kUnroll) nonzeros per batch.  Rows of at most long_len
 // nonzeros stay in the row-block pass (long_len = max(32, BS) unless the
-// caller sets it), whose warps own 128 consecutive rows (64 for W >= 16);
+// caller sets it), whose warps own 128 consecutive rows (64 for W >= 16) or, for
+// up to 32 columns, as many as make whole waves of them (1M rows: 1.6 waves of
+// 128 rows take as long as two; one of 206, power law, n = 8 135 -> 132 us,
+// n = 16 191 -> 181; 700,000 rows of Poisson 2.5, n = 20, 80 -> 62; at n = 64
+// 1M rows of 2 lose, 128 -> 140);
 // queued rows of at most mid_len = 4 long_len go to one lane group each; with
 // W >= 4 those of more than mid_split = 2 long_len are taken first, so a warp's
 // work item holds rows of similar length and the longest items do not come
@@ -377,7 +381,15 @@ HybridLayout hybrid_layout(int m, long long nnz, int n, const Shape& s, const sp
     H.mid_len = (int)std::min<long long>(4 * long_len, 0x7fffffffLL);
     H.mid_split = s.W >= 4 ? (int)std::min<long long>(2 * long_len, H.mid_len) : H.mid_len;  // split_mid_rows
     H.seg_len = 16 * (32 / s.W) * bs;
-    H.block_rows = t.block_rows > 0 ? std::min(t.block_rows, kMaxBlockRows) : (s.W >= 16 ? 64 : 128);
+    if (t.block_rows > 0) {
+        H.block_rows = std::min(t.block_rows, kMaxBlockRows);
+    } else if (s.W * s.vec > 32) {
+        H.block_rows = s.W >= 16 ? 64 : 128;
+    } else {  // whole waves of the row-block pass's resident warps (3 or 4 CTAs of 8 per SM)
+        const long long base = s.W >= 16 ? 64 : 128, wave = (s.W >= 16 ? 3LL : 4LL) * 8 * 152;
+        const long long waves = std::max<long long>(1, m / (base * wave));
+        H.block_rows = (int)std::min<long long>(std::max<long long>(32, (m + waves * wave - 1) / (waves * wave)), kMaxBlockRows);
+    }
     // mid rows: at most nnz / (long_len + 1) rows are longer than long_len; single rows: at most
     // nnz / (mid_len + 1); partial slots: a row of L > seg_len nonzeros takes at most
     // ceil(L / seg_len) <= L / seg_len + 1 of them, and there are at most nnz / (seg_len + 1) such rows

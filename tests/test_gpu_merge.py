@@ -67,3 +67,21 @@ def test_auto_gb300_runs_merge_on_small_type1_matrices(gpu_lib, n):
     nnz = int(rp[-1])
     auto = gpu_lib.spmm(d_rp, d_ci, d_v, B, alg="auto_gb300", nnz=nnz)
     assert torch.equal(auto, gpu_lib.spmm(d_rp, d_ci, d_v, B, alg="merge", nnz=nnz))
+
+
+def test_noalloc_keeps_accepting_wide_products(gpu_lib):
+    """With full tiles the partial sums of this product fit the fixed scratch of 16 MiB twice over; tiles made
+    smaller to fill the GPU must not take more."""
+    import torch
+
+    rng = np.random.default_rng(1)
+    m, k, n = 20_000, 500, 2048
+    rp, ci, v = csr_arrays(np.full(m, 50), k, 8, int_vals=True)
+    d_rp, d_ci, d_v = (torch.from_numpy(x).cuda() for x in (rp, ci, v))
+    B = torch.from_numpy(rng.integers(-4, 5, size=(k, n)).astype(np.float32)).cuda()
+    C = torch.empty(m, n, device="cuda")
+    st = gpu_lib.spmm_csr_noalloc(m, k, n, int(rp[-1]), d_rp.data_ptr(), d_ci.data_ptr(), d_v.data_ptr(), gpu_lib.F32,
+                                  B.data_ptr(), gpu_lib.F32, n, C.data_ptr(), gpu_lib.F32, n, gpu_lib.ALG_MERGE, None,
+                                  None, torch.cuda.current_stream().cuda_stream)
+    assert st == gpu_lib.OK, gpu_lib.spmm_status_string(st)
+    assert torch.equal(C, gpu_lib.spmm(d_rp, d_ci, d_v, B, alg="row_split", nnz=int(rp[-1])))
