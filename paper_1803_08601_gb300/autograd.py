@@ -42,14 +42,17 @@ class CSRMatrix:
 
     def transpose_pattern(self):
         """(row_ptr_t, col_ind_t, perm, max_row_t) of A^T, built on first use."""
-        if self._t is None:
-            self.queue_transpose()
-            rpt, cit, perm, probe = self._t_queued
-            # the longest row is read on a stream of its own, which waits for the transpose only; the call
-            # returns once that stream is done, so the parts are complete for every stream from here on
-            self._t = (rpt, cit, perm, max_row_length(rpt, stream=probe))
-            self._t_queued = None
-        return self._t
+        t, queued = self._t, self._t_queued
+        if t is None:
+            if queued is None:
+                parts = csr_transpose(self.row_ptr, self.col_ind, self.k)
+                t = (*parts, max_row_length(parts[0]))
+            else:
+                # the longest row is read on a stream of its own, which waits for the transpose only; the call
+                # returns once that stream is done, so the parts are complete for every stream from here on
+                t = (*queued[:3], max_row_length(queued[0], stream=queued[3]))
+            self._t, self._t_queued = t, None
+        return t
 
     def spmm(self, vals, B, alg=ALG_AUTO_GB300, **kw):
         given = kw.pop("tuning", None)
