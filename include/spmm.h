@@ -233,6 +233,9 @@ int spmm_csr(int m, int k, int n, const int *row_ptr, const int *col_ind, const 
  * workspace: device memory of at least spmm_csr_workspace_size(...) bytes for
  * the merge-based algorithm (row split and SPMM_ALG_TILED need none); NULL
  * with workspace_bytes == 0 makes the call allocate it stream-ordered itself.
+ * A merge of n > 1 whose default tiles need more than it is lent takes larger
+ * ones (other sums of the same terms), as long as tiles of 2048 merge-path items
+ * (1024 for up to 8 lanes per row, the caller's items_per_subwarp where set) fit.
  * n == 1 (y = A x) runs the SpMV kernels of the chosen family: the row split
  * with tuning->lanes_per_row lanes per row (0: from the mean row length) and
  * the merge based with 4, 8 or 16 path items per thread
@@ -280,6 +283,9 @@ int spmm_csr_semiring(int m, int k, int n, long long nnz, const int *row_ptr, co
  * (PARTITIONSPMM of Algorithm 1, Section 4.2) and each tile's carry-out and
  * head partial rows that FIXCARRYOUT combines; for the hybrid row split, its
  * queues of long rows and their segments' partial sums.  0 for row split.
+ * For a given n and alg (other than the selectors, whose choice depends on the
+ * sizes) it does not fall as m or nnz grows: a buffer for the largest pattern
+ * serves every smaller one.
  * alg SPMM_ALG_AUTO is resolved with the heuristic first.  Returns 0 for
  * invalid arguments.
  */

@@ -249,14 +249,13 @@ struct MergeLayout {
     size_t off_limits, off_carry_row, off_head_row, off_carry, off_head, total;
 };
 
-MergeLayout merge_layout(int m, long long nnz, int n, long long items_per_tile, int warps) {
+MergeLayout merge_layout(long long num_tiles, int warps, int n) {
     MergeLayout L{};
-    const long long total = (long long)m + nnz;
-    L.num_tiles = (int)((total + items_per_tile - 1) / items_per_tile);
-    L.ctas = (L.num_tiles + warps - 1) / warps;
+    L.num_tiles = (int)num_tiles;
+    L.ctas = (int)((num_tiles + warps - 1) / warps);
     size_t off = 0;
     L.off_limits = off;
-    off = align256(off + (size_t)(L.num_tiles + 1) * sizeof(int2));
+    off = align256(off + ((size_t)L.num_tiles + 1) * sizeof(int2));
     L.off_carry_row = off;
     off = align256(off + (size_t)L.ctas * 4);
     L.off_head_row = off;
@@ -304,50 +303,117 @@ Shape unaligned_shape(const Shape& base, int n, int tb, int tc, const void* B, l
     return s;
 }
 
-// Merge-path items per lane group of merge_kernel_narrow: tiles of kNarrowTile
-// items, or smaller ones that make one or two whole waves of its persistent
-// CTAs (6 per SM) where kNarrowTile would make at most two.  400,000 rows of
-// Poisson 2.5, n = 32: 1.5 waves of 1024 items 47 us, 2 of 768 42 us.
-int narrow_items(long long total, int groups) {
-    const long long wave = 6 * 152;
-    long long items = kNarrowTile;
-    if (total < wave * kNarrowTile * 2) {
-        const long long waves = total < wave * kNarrowTile * 5 / 8 ? 1 : 2;
-        items = std::max<long long>(128, (total + waves * wave - 1) / (waves * wave));
-    }
-    return std::max(4, (int)((items + groups - 1) / groups));
+// Tiles of a merge: merge-path items in each, tiles per CTA, and Shape::ips,
+// which is not 0 for the narrow kernel only.
+struct MergeTiles {
+    long long items;
+    int warps, ips;
+};
+
+MergeLayout merge_layout(int m, long long nnz, int n, const MergeTiles& t) {
+    return merge_layout(((long long)m + nnz + t.items - 1) / t.items, t.warps, n);
 }
 
-// Merge-path items per tile; sets s->ips, which is not 0 for the narrow kernel
-// only.  The caller's items_per_subwarp counts per lane group of a block of 256
-// threads (128 for up to 8 lanes per row), for the tiles of a whole CTA.  By
-// default a warp of merge_kernel takes about kMergeTile items, so that the
-// tiles make whole waves of the warps that the GPU runs at once (28 or 32 per
-// SM): a wave filled to a tenth costs as much as a full one.  300,000 rows of
-// Poisson 8, n = 128: 1.08 waves of 512 items 190 us, one wave of 555 147 us.
-// Where the partial sums are large (over 8 MiB) no tile is smaller than the full
-// one, so that a workspace of 16 MiB fits whatever it fitted with full tiles.
+// How many tiles a merge of `total` items makes by default, at most.  The number
+// does not fall as total grows: the bound of spmm_csr_workspace_size rests on it.
+//
+// merge_kernel_narrow: tiles of kNarrowTile items, or smaller ones that make one
+// or two whole waves of its persistent CTAs (6 per SM) where kNarrowTile would
+// make at most two.  400,000 rows of Poisson 2.5, n = 32: 1.5 waves of 1024
+// items 47 us, 2 of 768 42 us.
+constexpr long long kNarrowWave = 6 * 152;
+long long narrow_tiles(long long total) {
+    if (total >= 2 * kNarrowWave * kNarrowTile) return (total + kNarrowTile - 1) / kNarrowTile;
+    return std::min((total + 127) / 128, (total < kNarrowWave * kNarrowTile * 5 / 8 ? 1 : 2) * kNarrowWave);
+}
+
+// merge_kernel: a warp takes about kMergeTile items, so that the tiles make whole
+// waves of the warps that the GPU runs at once (28 or 32 per SM): a wave filled
+// to a tenth costs as much as a full one.  300,000 rows of Poisson 8, n = 128:
+// 1.08 waves of 512 items 190 us, one wave of 555 147 us.
 constexpr int kMergeTile = 512;
-long long merge_tile(int m, long long nnz, int n, const spmm_tuning_t* t, int sv, Shape* s) {
-    const int groups = (s->W >= 16 ? 256 : 128) / s->W;
-    const int asked = t && t->items_per_subwarp > 0 ? std::min(std::max(t->items_per_subwarp, 4), 4096) : 0;
-    const long long total = (long long)m + nnz;
-    s->ips = 0;
-    if (merge_narrow(m, nnz, *s)) {
-        const bool large = std::max(total / kNarrowTile, 2LL * 6 * 152) * n * 8 > (8LL << 20);
-        s->ips = asked ? asked : large ? kNarrowTile / groups : narrow_items(total, groups);
-        auto smem = [&]() -> size_t {
-            if (sv == 4) return s->vec == 1 ? merge_smem_vec<float, 1>(*s) : s->vec == 4 ? merge_smem_vec<float, 4>(*s) : merge_smem_vec<float, 8>(*s);
-            return s->vec == 1 ? merge_smem_vec<__half, 1>(*s) : s->vec == 4 ? merge_smem_vec<__half, 4>(*s) : merge_smem_vec<__half, 8>(*s);
-        };
-        while (s->ips > 4 && smem() > kMaxSmem) s->ips = s->ips * 3 / 4;  // until the double-buffered staging fits
-        return (long long)groups * s->ips;
+long long warp_wave(int W) { return (W < 32 ? 28LL : 32LL) * 152; }
+long long warp_tiles(long long total, int W) {
+    const long long wave = kMergeTile * warp_wave(W);
+    return std::min((total + 63) / 64, std::max<long long>(1, (total + wave / 2) / wave) * warp_wave(W));
+}
+
+// Items of a full tile of a CTA: what the caller asks for (items_per_subwarp
+// counts per lane group of a block of 256 threads, 128 for up to 8 lanes per
+// row), else 8 per thread.  Rows of up to 8 lanes may run the narrow kernel,
+// whose double-buffered staging has to fit (sv: bytes of a value).
+long long full_tile(const spmm_tuning_t* t, const Shape& shape, int sv) {
+    Shape s = shape;
+    const int groups = (s.W >= 16 ? 256 : 128) / s.W;
+    s.ips = t && t->items_per_subwarp > 0 ? std::min(std::max(t->items_per_subwarp, 4), 4096) : 8 * s.W;
+    auto smem = [&]() -> size_t {
+        if (sv == 4) return s.vec == 1 ? merge_smem_vec<float, 1>(s) : s.vec == 4 ? merge_smem_vec<float, 4>(s) : merge_smem_vec<float, 8>(s);
+        return s.vec == 1 ? merge_smem_vec<__half, 1>(s) : s.vec == 4 ? merge_smem_vec<__half, 4>(s) : merge_smem_vec<__half, 8>(s);
+    };
+    while (s.W <= 8 && s.ips > 4 && smem() > kMaxSmem) s.ips = s.ips * 3 / 4;
+    return (long long)groups * s.ips;
+}
+
+// Workspace of a merge of full tiles, one entry each: a merge whose caller lends
+// this much runs.
+size_t full_tiles_bytes(int m, long long nnz, int n, const spmm_tuning_t* t, const Shape& s, int sv) {
+    return merge_layout(m, nnz, n, MergeTiles{full_tile(t, s, sv), 1, 0}).total;
+}
+
+// The default tiles.  Where their partial sums are large (over 8 MiB) they are
+// full ones, or whole waves rounded down.
+MergeTiles merge_tiles(int m, long long nnz, int n, const spmm_tuning_t* t, const Shape& s, int sv) {
+    const bool asked = t && t->items_per_subwarp > 0;
+    const long long total = (long long)m + nnz, full = full_tile(t, s, sv);
+    if (merge_narrow(m, nnz, s)) {
+        const int groups = kNarrowThreads / s.W;
+        const bool large = std::max(total / kNarrowTile, 2 * kNarrowWave) * n * 8 > (8LL << 20);
+        const long long tiles = std::max<long long>(1, narrow_tiles(total));
+        const long long items = asked || large ? full : std::max<long long>(128, (total + tiles - 1) / tiles);
+        const int ips = std::max(4, (int)((items + groups - 1) / groups));
+        return {(long long)groups * ips, 1, ips};
     }
-    if (asked) return ((long long)groups * asked + kMergeWarps - 1) / kMergeWarps;
-    const long long per_wave = (s->W < 32 ? 28LL : 32LL) * 152, wave = kMergeTile * per_wave;
-    long long tiles = std::max<long long>(1, (total + wave / 2) / wave) * per_wave;
-    if (tiles / kMergeWarps * n * 8 > (8LL << 20)) tiles = total / wave * per_wave;  // large: rounded down
-    return tiles == 0 ? kMergeTile : std::max<long long>(64, (total + tiles - 1) / tiles);
+    if (asked) return {(full + kMergeWarps - 1) / kMergeWarps, kMergeWarps, 0};
+    const long long wave = kMergeTile * warp_wave(s.W);
+    long long tiles = std::max<long long>(1, (total + wave / 2) / wave) * warp_wave(s.W);
+    if (tiles / kMergeWarps * n * 8 > (8LL << 20)) tiles = total / wave * warp_wave(s.W);
+    return {tiles == 0 ? kMergeTile : std::max<long long>(64, (total + tiles - 1) / tiles), kMergeWarps, 0};
+}
+
+// Fits the default tiles to a lent workspace of `bytes`: the smallest tiles not
+// below them that it holds.  False where it holds neither them nor full tiles of
+// one entry each.
+bool fit_merge_tiles(int m, long long nnz, int n, const spmm_tuning_t* t, const Shape& s, int sv, size_t bytes,
+                     MergeTiles* tiles) {
+    const int step = tiles->ips > 0 ? kNarrowThreads / s.W : 1;  // the narrow kernel's are whole lane groups
+    auto fits = [&](long long steps) {
+        return merge_layout(m, nnz, n, MergeTiles{steps * step, tiles->warps, 0}).total <= bytes;
+    };
+    long long lo = tiles->items / step, hi = full_tile(t, s, sv) / step;
+    if (fits(lo)) return true;
+    if (hi <= lo || full_tiles_bytes(m, nnz, n, t, s, sv) > bytes) return false;
+    while (hi - lo > 1) {  // hi fits, lo does not
+        const long long mid = lo + (hi - lo) / 2;
+        (fits(mid) ? hi : lo) = mid;
+    }
+    tiles->items = hi * step;
+    if (tiles->ips > 0) tiles->ips = (int)hi;
+    return true;
+}
+
+// Workspace for a merge with lanes like those of s, of at most m rows and nnz
+// nonzeros: it does not fall as either grows, as the default tiles alone would,
+// whose kernel and waves change with both.  It holds the default tiles of either
+// kernel, up to 15/4 of the workspace of full ones (up to just that above 8 MiB).
+size_t merge_bound(int m, long long nnz, int n, const spmm_tuning_t* t, const Shape& s) {
+    const long long total = (long long)m + nnz, full = full_tile(t, s, 4);
+    const bool asked = t && t->items_per_subwarp > 0;
+    const long long quarter = (full + kMergeWarps - 1) / kMergeWarps;
+    const size_t full_bytes = full_tiles_bytes(m, nnz, n, t, s, 4);
+    size_t tiled = merge_layout(asked ? (total + quarter - 1) / quarter : warp_tiles(total, s.W), kMergeWarps, n).total;
+    if (s.W <= 8) tiled = std::max(tiled, merge_layout(asked ? (total + full - 1) / full : narrow_tiles(total), 1, n).total);
+    const size_t most = std::max(full_bytes, std::min<size_t>(full_bytes / 4 * 15, 8u << 20));
+    return align256(std::max(full_bytes, std::min(tiled, most)));
 }
 
 // Hybrid row split (SPMM_ALG_ROW_SPLIT_HYBRID).  A lane group of W lanes
@@ -659,8 +725,12 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
 
     // merge based: partition, compute, fix-up
     const int spmv_t = spmv_items(&t_eff);
-    const long long ipt = spmv ? (long long)kThreads * spmv_t : merge_tile(m, nnz, n, &t_eff, dtype_size(vals_type), &shape);
-    const MergeLayout lay = merge_layout(m, nnz, n, ipt, spmv || shape.ips > 0 ? 1 : kMergeWarps);
+    const int sv = dtype_size(vals_type);
+    MergeTiles tiles = spmv ? MergeTiles{(long long)kThreads * spmv_t, 1, 0} : merge_tiles(m, nnz, n, &t_eff, shape, sv);
+    if (workspace && !spmv && !fit_merge_tiles(m, nnz, n, &t_eff, shape, sv, workspace_bytes, &tiles))
+        return SPMM_ERR_WORKSPACE;
+    const MergeLayout lay = merge_layout(m, nnz, n, tiles);
+    shape.ips = tiles.ips;
     bool own = false;
     unsigned char* ws = static_cast<unsigned char*>(workspace);
     if (!ws) {
@@ -699,7 +769,7 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
     if (!spmv && shape.vec == 1 && shape.ips == 0)
         shape = unaligned_shape(shape, n, b_type, c_type, B, ldb, C, ldc, tuning);
     ma.slabs = shape.slabs;
-    st = spmm_merge_partition(m, nnz, row_ptr, (int)ipt, lay.num_tiles, reinterpret_cast<int*>(ws + lay.off_limits),
+    st = spmm_merge_partition(m, nnz, row_ptr, (int)tiles.items, lay.num_tiles, reinterpret_cast<int*>(ws + lay.off_limits),
                               stream);
     if (st == SPMM_OK) st = cuda_status(spmv ? L->spmv_merge(ma, spmv_t, s) : L->merge(ma, shape, sm_count(), s));
     if (st == SPMM_OK && lay.ctas > 1) st = cuda_status(L->fixup(ma, lay.ctas, s));
@@ -819,14 +889,11 @@ size_t spmm_csr_workspace_size(int m, int k, int n, long long nnz, int alg, int 
             if (slabs) t.column_slabs = slabs;
             Shape s;
             if (!shape_for(n, vec, &t, &s)) return 0;
-            const long long items = merge_tile(m, nnz, n, &t, 4, &s);
-            const size_t need = merge_layout(m, nnz, n, items, s.ips > 0 ? 1 : kMergeWarps).total;
-            if (need > best) best = need;
+            best = std::max(best, merge_bound(m, nnz, n, &t, s));
         }
     }
     if (n == 1) {  // the SpMV form's tiles
-        const size_t need = merge_layout(m, nnz, n, (long long)kThreads * spmv_items(tuning), 1).total;
-        if (need > best) best = need;
+        best = std::max(best, merge_layout(m, nnz, n, MergeTiles{(long long)kThreads * spmv_items(tuning), 1, 0}).total);
     }
     return best;
 }
