@@ -164,15 +164,6 @@ TRAFFIC_COMMAND = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,lts
                    "--no-clocks")
 
 
-def auto_gb300_runs(pkg, pick, nnz, max_row, n):
-    """The family a float32 SPMM_ALG_AUTO_GB300 call runs when the selector's rule names `pick` (include/spmm.h)."""
-    if pick != pkg.ALG_ROW_SPLIT_HYBRID:
-        return pick
-    type1 = max_row > 1024 and max_row * 8192 >= nnz
-    ahead = n > 1 and n % 4 == 0 and ((n <= 16 and nnz >= 8 << 20) if type1 else (n <= 64 and nnz >= 1_500_000))
-    return pick if ahead else pkg.ALG_MERGE
-
-
 def sources_sha256(paths):
     import hashlib
 
@@ -468,9 +459,8 @@ def main():
     d_C = {n: torch.empty((m, n), dtype=torch.float32, device=dev) for n in ns}
     max_row = pkg.max_row_length(d_rp)  # measured once; passed to the GB300 selector as a hint
     paper_pick = {n: pkg.spmm_select_alg(m, nnz, 0.0) for n in ns}
-    gb300_pick = {n: pkg.spmm_select_alg_gb300(m, nnz, max_row, n, pkg.F32) for n in ns}
-    gb300_runs = {n: auto_gb300_runs(pkg, gb300_pick[n], nnz, max_row, n) for n in ns}
-    alg_of = {n: {"auto": paper_pick[n], "auto_gb300": gb300_runs[n]}.get(args.alg, pkg.alg_code(args.alg)) for n in ns}
+    gb300_pick = {n: pkg.spmm_auto_gb300_alg(m, nnz, max_row, n, pkg.F32) for n in ns}
+    alg_of = {n: {"auto": paper_pick[n], "auto_gb300": gb300_pick[n]}.get(args.alg, pkg.alg_code(args.alg)) for n in ns}
     tuning_ws = json.loads(args.tuning) if args.tuning else None
     ws_bytes = max(pkg.workspace_size(m, k, n, nnz, al, tuning=tuning_ws)
                    for n in ns for al in (pkg.ALG_MERGE, pkg.ALG_ROW_SPLIT_HYBRID))
@@ -881,7 +871,7 @@ def plain_latency(pkg, torch, flush, stream, steps):
     C = torch.empty((a.m, n), device=dev)
     lmax = pkg.max_row_length(rp)
     tun = {"max_row_len": lmax}
-    alg = pkg.spmm_select_alg_gb300(a.m, a.nnz, lmax, n, pkg.F32)
+    alg = pkg.spmm_auto_gb300_alg(a.m, a.nnz, lmax, n, pkg.F32)
     ws_b = max(pkg.workspace_size(a.m, a.k, n, a.nnz, al) for al in (pkg.ALG_MERGE, pkg.ALG_ROW_SPLIT_HYBRID))
     ws = torch.empty(max(ws_b, 256), dtype=torch.uint8, device=dev)
 
@@ -1031,7 +1021,7 @@ def run_sweep(args):
                                  pkg.workspace_size(m, k, n, total, "hybrid")), dtype=torch.uint8, device=dev)
             row = {"sweep": "aspect", "m": m, "k": k, "nnz": total, "n": n,
                    "paper_pick": name[pkg.spmm_select_alg(m, total, 0.0)],
-                   "gb300_pick": name[pkg.spmm_select_alg_gb300(m, total, k, n, pkg.F32)]}
+                   "gb300_pick": name[pkg.spmm_auto_gb300_alg(m, total, k, n, pkg.F32)]}
             for alg in ("row_split", "merge", "hybrid"):
                 r = reps if (alg == "merge" or k <= (1 << 16)) else 1  # very long rows: one timed run
                 t = _time(torch, lambda: pkg.spmm(rp, ci, v, B, alg=alg, out=C, nnz=total, workspace=ws),
@@ -1083,7 +1073,7 @@ def run_sweep(args):
             lmax = per_row
             tun = {"max_row_len": lmax}
             row = {"sweep": "density", "m": mk, "k": mk, "per_row": per_row, "density": per_row / mk,
-                   "nnz": per_row * mk, "n": n, "gb300_pick": name[pkg.spmm_select_alg_gb300(mk, per_row * mk, lmax, n, pkg.F32)]}
+                   "nnz": per_row * mk, "n": n, "gb300_pick": name[pkg.spmm_auto_gb300_alg(mk, per_row * mk, lmax, n, pkg.F32)]}
             t = _time(torch, lambda: pkg.spmm(rp, ci, v, B, alg="auto_gb300", out=C, nnz=per_row * mk, tuning=tun),
                       flush, stream, reps)
             row["spmm"] = {"ms": t, "gflops": 2.0 * per_row * mk * n / t / 1e6}
@@ -1168,7 +1158,7 @@ def run_selector_sweep(pkg, torch, dev, flush, stream, reps):
                                    stream, r)
                 best = min(t.values())
                 paper = name[pkg.spmm_select_alg(m, nnz, 0.0)]
-                gb300 = name[pkg.spmm_select_alg_gb300(m, nnz, lmax, n, pkg.F32)]
+                gb300 = name[pkg.spmm_auto_gb300_alg(m, nnz, lmax, n, pkg.F32)]
                 print(json.dumps({"sweep": "selector", "family": family, "mean_row": nnz / m, "max_row": lmax,
                                   "n": n, "nnz": nnz, "row_split_ms": t["row_split"], "merge_ms": t["merge"],
                                   "hybrid_ms": t["hybrid"],
@@ -1202,7 +1192,7 @@ def run_spmv_sweep(pkg, torch, dev, flush, stream, reps):
         row = {"sweep": "spmv", "matrix": label, "m": m, "k": k, "nnz": nnz, "max_row": lmax,
                "compulsory_bytes": comp, "peak_gbs": peak, "peak_source": peak_src,
                "paper_pick": name[pkg.spmm_select_alg(m, nnz, 0.0)],
-               "gb300_pick": name[pkg.spmm_select_alg_gb300(m, nnz, lmax, 1, pkg.F32)]}
+               "gb300_pick": name[pkg.spmm_auto_gb300_alg(m, nnz, lmax, 1, pkg.F32)]}
         tun = {"max_row_len": lmax}
         ref = None
         for alg in ("row_split", "merge", "auto", "auto_gb300"):

@@ -165,14 +165,21 @@ int spmm_select_alg(int m, long long nnz, double threshold);
  *     of 512 bytes or more and 3 for 256-511 bytes; SPMM_ALG_ROW_SPLIT
  *     otherwise (measured crossovers for uniform and Poisson row lengths).
  * m == 0 returns row split.
- * SPMM_ALG_AUTO_GB300 follows this rule, except that it runs the merge based
- * algorithm where the rule names the hybrid row split, unless n > 1, rows of B
- * are whole 16-byte vectors and the matrix is large: 2^23 nonzeros and rows of B
- * of at most 64 bytes for a Type 1 matrix, 1.5 million nonzeros and at most 256
- * bytes otherwise.  The merge kernel has overtaken the hybrid elsewhere since
- * the sweeps.
+ * SPMM_ALG_AUTO_GB300 follows this rule except where it names the hybrid row
+ * split: spmm_auto_gb300_alg gives the family that a call runs.
  */
 int spmm_select_alg_gb300(int m, long long nnz, long long max_row_len, int n, int b_type);
+
+/*
+ * The family (SPMM_ALG_ROW_SPLIT, SPMM_ALG_MERGE or SPMM_ALG_ROW_SPLIT_HYBRID)
+ * that SPMM_ALG_AUTO_GB300 runs for these sizes, pure host function: that of
+ * spmm_select_alg_gb300, but merge in the place of the hybrid, which the merge
+ * kernel has overtaken since the sweeps, unless n > 1, rows of B are whole
+ * 16-byte vectors and the matrix is large: 2^23 nonzeros and rows of B of at
+ * most 64 bytes for a Type 1 matrix, 1.5 million nonzeros and at most 256 bytes
+ * otherwise.
+ */
+int spmm_auto_gb300_alg(int m, long long nnz, long long max_row_len, int n, int b_type);
 
 /*
  * Expected reuse of one staged B row under SPMM_ALG_TILED: the rows of A per

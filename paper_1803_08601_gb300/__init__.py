@@ -62,6 +62,7 @@ _SIGNATURES = {
     "spmm_launch_count": ([], _ll),
     "spmm_select_alg": ([_i, _ll, _d], _i),
     "spmm_select_alg_gb300": ([_i, _ll, _ll, _i, _i], _i),
+    "spmm_auto_gb300_alg": ([_i, _ll, _ll, _i, _i], _i),
     "spmm_gather_probe": ([_vp, _ll, _i, _vp, _ll, _vp, _vp], _i),
     "spmm_default_column_slabs": ([_i, _i, _i, _i], _i),
     "spmm_tiled_reuse": ([_i, _i, _ll, _i, _i], _d),
@@ -134,6 +135,11 @@ def spmm_select_alg(m: int, nnz: int, threshold: float = 0.0) -> int:
 
 def spmm_select_alg_gb300(m: int, nnz: int, max_row_len: int, n: int, b_type: int = F32) -> int:
     return load().spmm_select_alg_gb300(m, nnz, max_row_len, n, b_type)
+
+
+def spmm_auto_gb300_alg(m: int, nnz: int, max_row_len: int, n: int, b_type: int = F32) -> int:
+    """The family that ALG_AUTO_GB300 runs for these sizes."""
+    return load().spmm_auto_gb300_alg(m, nnz, max_row_len, n, b_type)
 
 
 def spmm_tiled_reuse(m: int, k: int, nnz: int, n: int, b_type: int = F32) -> float:

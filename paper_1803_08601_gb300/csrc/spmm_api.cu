@@ -117,27 +117,6 @@ int resolve_alg(int alg, int m, long long nnz, const spmm_tuning_t* t) {
     return spmm_select_alg(m, nnz, threshold_of(t));
 }
 
-// What SPMM_ALG_AUTO_GB300 runs: the family of spmm_select_alg_gb300, with merge
-// in the place of the hybrid row split wherever merge_kernel, which is newer
-// than the sweeps behind that rule, has overtaken it.  With rows of B in whole
-// 16-byte vectors the hybrid stays ahead for rows of up to 64 bytes of large
-// Type 1 matrices and, below 3 nonzeros per row, for rows of up to 256 bytes of
-// large ones.  Measured on GB300, hybrid / merge (us): power law 1M (15.9M
-// nonzeros), n = 8 134 / 167, n = 13 346 / 225, n = 32 296 / 274; 300,000 rows
-// of it (4.8M), n = 8 62 / 62, n = 32 104 / 82; graph of 200,000 nodes, n = 8
-// 64 / 45; 1M rows of 2, n = 32 75 / 86, n = 64 129 / 131, n = 100 304 / 223;
-// 400,000 of Poisson 2.5, n = 32 46 / 42.  With n = 1 merge is the SpMV kernel,
-// the hybrid one lane per row: 1M power law, 124 / 94.
-int route_gb300(int m, long long nnz, long long max_row_len, int n, int b_type) {
-    const int a = spmm_select_alg_gb300(m, nnz, max_row_len, n, b_type);
-    if (a != SPMM_ALG_ROW_SPLIT_HYBRID) return a;
-    const long long row_bytes = (long long)n * dtype_size(b_type);
-    const bool type1 = max_row_len > 1024 && max_row_len * 8192 >= nnz;
-    const bool ahead = n > 1 && row_bytes % 16 == 0 &&
-                       (type1 ? row_bytes <= 64 && nnz >= (8LL << 20) : row_bytes <= 256 && nnz >= 1500000);
-    return ahead ? a : (int)SPMM_ALG_MERGE;
-}
-
 // row_ptr[i] -= base for i < count: a row chunk's offsets made to start at 0.
 __global__ void rebase_kernel(int* __restrict__ row_ptr, int count, int base) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -664,7 +643,7 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
         if (st != SPMM_OK) return st;
     }
     Shape shape;
-    if (alg == SPMM_ALG_AUTO_GB300) alg = route_gb300(m, nnz, lmax, n, b_type);
+    if (alg == SPMM_ALG_AUTO_GB300) alg = spmm_auto_gb300_alg(m, nnz, lmax, n, b_type);
     const int a = resolve_alg(alg, m, nnz, tuning);
     spmm_tuning_t t_eff = tuning ? *tuning : spmm_tuning_t{};
     if (t_eff.column_slabs <= 0 && t_eff.lanes_per_row <= 0) t_eff.column_slabs = default_slabs(a, k, n, b_type, L->plus_times);
@@ -837,6 +816,27 @@ int spmm_select_alg_gb300(int m, long long nnz, long long max_row_len, int n, in
     return d < threshold ? SPMM_ALG_MERGE : SPMM_ALG_ROW_SPLIT;
 }
 
+// What SPMM_ALG_AUTO_GB300 runs: the family of spmm_select_alg_gb300, with merge
+// in the place of the hybrid row split wherever merge_kernel, which is newer
+// than the sweeps behind that rule, has overtaken it.  With rows of B in whole
+// 16-byte vectors the hybrid stays ahead for rows of up to 64 bytes of large
+// Type 1 matrices and, below 3 nonzeros per row, for rows of up to 256 bytes of
+// large ones.  Measured on GB300, hybrid / merge (us): power law 1M (15.9M
+// nonzeros), n = 8 134 / 167, n = 13 346 / 225, n = 32 296 / 274; 300,000 rows
+// of it (4.8M), n = 8 62 / 62, n = 32 104 / 82; graph of 200,000 nodes, n = 8
+// 64 / 45; 1M rows of 2, n = 32 75 / 86, n = 64 129 / 131, n = 100 304 / 223;
+// 400,000 of Poisson 2.5, n = 32 46 / 42.  With n = 1 merge is the SpMV kernel,
+// the hybrid one lane per row: 1M power law, 124 / 94.
+int spmm_auto_gb300_alg(int m, long long nnz, long long max_row_len, int n, int b_type) {
+    const int a = spmm_select_alg_gb300(m, nnz, max_row_len, n, b_type);
+    if (a != SPMM_ALG_ROW_SPLIT_HYBRID) return a;
+    const long long row_bytes = (long long)n * (dtype_size(b_type) ? dtype_size(b_type) : 4);
+    const bool type1 = max_row_len > 1024 && max_row_len * 8192 >= nnz;
+    const bool ahead = n > 1 && row_bytes % 16 == 0 &&
+                       (type1 ? row_bytes <= 64 && nnz >= (8LL << 20) : row_bytes <= 256 && nnz >= 1500000);
+    return ahead ? a : (int)SPMM_ALG_MERGE;
+}
+
 double spmm_tiled_reuse(int m, int k, long long nnz, int n, int b_type) {
     if (m <= 0 || k <= 0 || n <= 0 || nnz <= 0 || dtype_size(b_type) == 0) return 0.0;
     const long long chunks = ((long long)n + 16 / dtype_size(b_type) - 1) / (16 / dtype_size(b_type));
@@ -987,7 +987,7 @@ static int host_products(int m, int k, const int* row_ptr, const int* col_ind, c
     for (size_t q = 0; q < prods.size(); ++q) {
         Prod& p = P[q];
         p.n = n_of[prods[q]];
-        p.alg = alg_req == SPMM_ALG_AUTO_GB300 ? route_gb300(m, nnz, t.max_row_len, p.n, b_type) : alg_req;
+        p.alg = alg_req == SPMM_ALG_AUTO_GB300 ? spmm_auto_gb300_alg(m, nnz, t.max_row_len, p.n, b_type) : alg_req;
         p.alg = resolve_alg(p.alg, m, nnz, &t);
         p.ldb_d = (p.n + vb - 1) / vb * vb;
         p.ldc_d = (p.n + vc - 1) / vc * vc;

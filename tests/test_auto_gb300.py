@@ -1,0 +1,31 @@
+"""The family that SPMM_ALG_AUTO_GB300 runs, and that the library names for it."""
+import pytest
+
+import paper_1803_08601_gb300 as pkg
+from test_workspace import problem
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("m,nnz,longest,n", [(4000, 20_000, 3000, 1), (4000, 20_000, 3000, 8), (4000, 20_000, 3000, 64),
+                                             (600_000, 9_600_000, 1_000_000, 8), (600_000, 9_600_000, 1_000_000, 32),
+                                             (900_000, 1_800_000, 2, 32), (30_000, 60_000, 2, 32),
+                                             (30_000, 300_000, 10, 32), (30_000, 300_000, 10, 8)])
+def test_a_call_runs_the_family_that_is_named(gpu_lib, m, nnz, longest, n):
+    """By the bits and the launches of a forced call: 1 for the row split, 2 for the hybrid, 3 for merge.  The
+    large skewed matrix at n = 8 has to stay with the hybrid."""
+    import torch
+
+    rp, ci, v, B = problem(torch, m, 1000, n, nnz)
+    if longest > nnz // m:  # the first row takes what the others give up
+        rp[1:] = (longest + torch.arange(m, device="cuda", dtype=torch.int64) * (nnz - longest) // (m - 1)).int()
+    alg = gpu_lib.spmm_auto_gb300_alg(m, nnz, longest, n, gpu_lib.F32)
+    if n == 8 and m == 600_000:
+        assert alg == gpu_lib.ALG_ROW_SPLIT_HYBRID
+    v = torch.randn(nnz, device="cuda")
+    counts, C = [], []
+    for a in (pkg.ALG_AUTO_GB300, alg):
+        before = gpu_lib.spmm_launch_count()
+        C.append(gpu_lib.spmm(rp, ci, v, B, alg=a, nnz=nnz, tuning=dict(max_row_len=longest)))
+        counts.append(gpu_lib.spmm_launch_count() - before)
+    assert counts[0] == counts[1] == {pkg.ALG_ROW_SPLIT: 1, pkg.ALG_ROW_SPLIT_HYBRID: 2, pkg.ALG_MERGE: 3}[alg]
+    assert torch.equal(*C)
