@@ -177,7 +177,8 @@ int spmm_select_alg_gb300(int m, long long nnz, long long max_row_len, int n, in
  * kernel has overtaken since the sweeps, unless n > 1, rows of B are whole
  * 16-byte vectors and the matrix is large: 2^23 nonzeros and rows of B of at
  * most 64 bytes for a Type 1 matrix, 1.5 million nonzeros and at most 256 bytes
- * otherwise.
+ * otherwise.  A call that is lent too small a workspace for merge, but one that
+ * the hybrid fits, runs the hybrid.
  */
 int spmm_auto_gb300_alg(int m, long long nnz, long long max_row_len, int n, int b_type);
 

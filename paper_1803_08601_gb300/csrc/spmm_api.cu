@@ -643,7 +643,11 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
         if (st != SPMM_OK) return st;
     }
     Shape shape;
-    if (alg == SPMM_ALG_AUTO_GB300) alg = spmm_auto_gb300_alg(m, nnz, lmax, n, b_type);
+    bool for_hybrid = false;  // merge in the place of the hybrid that the selector names
+    if (alg == SPMM_ALG_AUTO_GB300) {
+        alg = spmm_auto_gb300_alg(m, nnz, lmax, n, b_type);
+        for_hybrid = alg == SPMM_ALG_MERGE && spmm_select_alg_gb300(m, nnz, lmax, n, b_type) == SPMM_ALG_ROW_SPLIT_HYBRID;
+    }
     const int a = resolve_alg(alg, m, nnz, tuning);
     spmm_tuning_t t_eff = tuning ? *tuning : spmm_tuning_t{};
     if (t_eff.column_slabs <= 0 && t_eff.lanes_per_row <= 0) t_eff.column_slabs = default_slabs(a, k, n, b_type, L->plus_times);
@@ -706,8 +710,13 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
     const int spmv_t = spmv_items(&t_eff);
     const int sv = dtype_size(vals_type);
     MergeTiles tiles = spmv ? MergeTiles{(long long)kThreads * spmv_t, 1, 0} : merge_tiles(m, nnz, n, &t_eff, shape, sv);
-    if (workspace && !spmv && !fit_merge_tiles(m, nnz, n, &t_eff, shape, sv, workspace_bytes, &tiles))
-        return SPMM_ERR_WORKSPACE;
+    if (workspace && !(spmv ? merge_layout(m, nnz, n, tiles).total <= workspace_bytes
+                            : fit_merge_tiles(m, nnz, n, &t_eff, shape, sv, workspace_bytes, &tiles))) {
+        if (!for_hybrid) return SPMM_ERR_WORKSPACE;
+        // a workspace sized for the family that spmm_select_alg_gb300 names holds that one
+        return run_spmm(L, m, k, n, nnz, row_ptr, col_ind, vals, vals_type, B, b_type, ldb, C, c_type, ldc,
+                        SPMM_ALG_ROW_SPLIT_HYBRID, tuning, workspace, workspace_bytes, d_status, stream);
+    }
     const MergeLayout lay = merge_layout(m, nnz, n, tiles);
     shape.ips = tiles.ips;
     bool own = false;
@@ -720,7 +729,7 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
         if (e != cudaSuccess) return SPMM_ERR_ALLOC;
         ws = static_cast<unsigned char*>(p);
         own = true;
-    } else if (workspace_bytes < lay.total || ((uintptr_t)ws % 256) != 0) {
+    } else if ((uintptr_t)ws % 256 != 0) {
         return SPMM_ERR_WORKSPACE;
     }
     MergeArgs ma{};

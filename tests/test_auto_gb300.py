@@ -29,3 +29,24 @@ def test_a_call_runs_the_family_that_is_named(gpu_lib, m, nnz, longest, n):
         counts.append(gpu_lib.spmm_launch_count() - before)
     assert counts[0] == counts[1] == {pkg.ALG_ROW_SPLIT: 1, pkg.ALG_ROW_SPLIT_HYBRID: 2, pkg.ALG_MERGE: 3}[alg]
     assert torch.equal(*C)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [1, 4, 8, 16])
+def test_a_workspace_for_the_selected_family_is_enough(gpu_lib, n):
+    """Sized for the hybrid that the selector names, where the call runs merge if it allocates for itself."""
+    import torch
+
+    m, nnz, longest = 3_000_000, 400_000, 200_000  # full merge tiles take more than the hybrid
+    rp, ci, v, B = problem(torch, m, 1000, n, nnz)
+    rp[1:] = (longest + torch.arange(m, device="cuda", dtype=torch.int64) * (nnz - longest) // (m - 1)).int()
+    named = gpu_lib.spmm_select_alg_gb300(m, nnz, longest, n, gpu_lib.F32)
+    assert named == gpu_lib.ALG_ROW_SPLIT_HYBRID
+    assert gpu_lib.spmm_auto_gb300_alg(m, nnz, longest, n, gpu_lib.F32) == gpu_lib.ALG_MERGE
+    ws = torch.empty(gpu_lib.workspace_size(m, 1000, n, nnz, named), dtype=torch.uint8, device="cuda")
+    hint = dict(max_row_len=longest)
+    C = gpu_lib.spmm(rp, ci, v, B, alg="auto_gb300", nnz=nnz, tuning=hint, workspace=ws)
+    assert torch.equal(C, gpu_lib.spmm(rp, ci, v, B, alg="merge", nnz=nnz))
+    with pytest.raises(gpu_lib.SpMMError) as e:
+        gpu_lib.spmm(rp, ci, v, B, alg="auto_gb300", nnz=nnz, tuning=hint, workspace=ws[:1024])
+    assert e.value.status == gpu_lib.ERR_WORKSPACE
