@@ -120,7 +120,8 @@ typedef struct {
     int block_rows;          /* SPMM_ALG_ROW_SPLIT_HYBRID: consecutive rows per warp in
                                 the row-block pass, 1-256 (larger values act as 256);
                                 0 selects 128, or 64 for >= 16 lanes per row, and for
-                                up to 32 columns as many as make whole waves of warps   */
+                                up to 32 columns, in one slab, as many as make whole
+                                waves of warps                                          */
 } spmm_tuning_t;
 
 /* Human-readable name of a status code (static storage).  The paper defines

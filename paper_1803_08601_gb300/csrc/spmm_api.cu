@@ -402,7 +402,9 @@ size_t merge_bound(int m, long long nnz, int n, const spmm_tuning_t* t, const Sh
 // up to 32 columns, as many as make whole waves of them (1M rows: 1.6 waves of
 // 128 rows take as long as two; one of 206, power law, n = 8 135 -> 132 us,
 // n = 16 191 -> 181; 700,000 rows of Poisson 2.5, n = 20, 80 -> 62; at n = 64
-// 1M rows of 2 lose, 128 -> 140);
+// 1M rows of 2 lose, 128 -> 140, and in two slabs 1.2M rows of 1, 115 -> 130).
+// From 1.75 on it is two waves: one of 246 rows takes longer than 1.9 of 128
+// (1.2M rows of 2, n = 32, 97 us against 89; of 1, 77 against 68);
 // queued rows of at most mid_len = 4 long_len go to one lane group each; with
 // W >= 4 those of more than mid_split = 2 long_len are taken first, so a warp's
 // work item holds rows of similar length and the longest items do not come
@@ -428,11 +430,11 @@ HybridLayout hybrid_layout(int m, long long nnz, int n, const Shape& s, const sp
     H.seg_len = 16 * (32 / s.W) * bs;
     if (t.block_rows > 0) {
         H.block_rows = std::min(t.block_rows, kMaxBlockRows);
-    } else if (s.W * s.vec > 32) {
+    } else if (s.W * s.vec > 32 || s.slabs > 1) {
         H.block_rows = s.W >= 16 ? 64 : 128;
     } else {  // whole waves of the row-block pass's resident warps (3 or 4 CTAs of 8 per SM)
         const long long base = s.W >= 16 ? 64 : 128, wave = (s.W >= 16 ? 3LL : 4LL) * 8 * 152;
-        const long long waves = std::max<long long>(1, m / (base * wave));
+        const long long waves = std::max<long long>(1, (m + base * wave / 4) / (base * wave));
         H.block_rows = (int)std::min<long long>(std::max<long long>(32, (m + waves * wave - 1) / (waves * wave)), kMaxBlockRows);
     }
     // mid rows: at most nnz / (long_len + 1) rows are longer than long_len; single rows: at most
