@@ -175,10 +175,17 @@ int spmm_select_alg_gb300(int m, long long nnz, long long max_row_len, int n, in
  * The family (SPMM_ALG_ROW_SPLIT, SPMM_ALG_MERGE or SPMM_ALG_ROW_SPLIT_HYBRID)
  * that SPMM_ALG_AUTO_GB300 runs for these sizes, pure host function: that of
  * spmm_select_alg_gb300, but merge in the place of the hybrid, which the merge
- * kernel has overtaken since the sweeps, unless n > 1, rows of B are whole
- * 16-byte vectors and the matrix is large: 2^23 nonzeros and rows of B of at
- * most 64 bytes for a Type 1 matrix, 1.5 million nonzeros and at most 256 bytes
- * otherwise.  A call that is lent too small a workspace for merge, but one that
+ * kernel has overtaken since the sweeps, unless n > 1 and one of these holds, with
+ * rows of B in whole 16-byte vectors:
+ *   - a Type 1 matrix, rows of B of at most 64 bytes and 6 million nonzeros, or of
+ *     at most 128 bytes in 16 bits and 4 million (not whole vectors: n = 2 and 12
+ *     million);
+ *   - otherwise, rows of B of at most 128 bytes and 1.5 million nonzeros (1 million
+ *     where d < 2.25); of at most 256 in 16 bits and 300,000 (any number where
+ *     d < 2.25); of at most 256 in 32 bits and 1.5 million (450,000 where d < 2.25,
+ *     1.1 million for 256 bytes); of 512 bytes or more (in 16 bits, below 640) and
+ *     520,000 rows.
+ * A call that is lent too small a workspace for merge, but one that
  * the hybrid fits, runs the hybrid.
  */
 int spmm_auto_gb300_alg(int m, long long nnz, long long max_row_len, int n, int b_type);

@@ -829,22 +829,31 @@ int spmm_select_alg_gb300(int m, long long nnz, long long max_row_len, int n, in
 
 // What SPMM_ALG_AUTO_GB300 runs: the family of spmm_select_alg_gb300, with merge
 // in the place of the hybrid row split wherever merge_kernel, which is newer
-// than the sweeps behind that rule, has overtaken it.  With rows of B in whole
-// 16-byte vectors the hybrid stays ahead for rows of up to 64 bytes of large
-// Type 1 matrices and, below 3 nonzeros per row, for rows of up to 256 bytes of
-// large ones.  Measured on GB300, hybrid / merge (us): power law 1M (15.9M
-// nonzeros), n = 8 134 / 167, n = 13 346 / 225, n = 32 296 / 274; 300,000 rows
-// of it (4.8M), n = 8 62 / 62, n = 32 104 / 82; graph of 200,000 nodes, n = 8
-// 64 / 45; 1M rows of 2, n = 32 75 / 86, n = 64 129 / 131, n = 100 304 / 223;
-// 400,000 of Poisson 2.5, n = 32 46 / 42.  With n = 1 merge is the SpMV kernel,
-// the hybrid one lane per row: 1M power law, 124 / 94.
+// than the sweeps behind that rule, has overtaken it.  The hybrid stays ahead for
+// rows of B in whole 16-byte vectors of large matrices, the more so the fewer
+// bytes a row has, in 16 bits and where rows of A are 1 or 2 nonzeros.  Measured
+// on GB300, hybrid / merge (us).  Power-law rows: 5.3M nonzeros, bf16 n = 16
+// 92 / 87, n = 64 157 / 178; 6.7M, n = 8 74 / 82, n = 32 120 / 109, bf16 n = 64
+// 165 / 214; 23.5M, n = 2 162 / 181, n = 8 177 / 228, n = 20 and up, 20 % behind;
+// 1.9M, everything behind.  Fewer than 3 per row: 1.2M rows of 2, n = 32 87 / 95,
+// n = 40 1.18 times, n = 64 150 / 160, n = 128 283 / 301, n = 100 1.3 behind;
+// 500,000 rows of 1, n = 40 52 / 59, n = 64 0.92 times, bf16 n = 128 68 / 87;
+// bf16 n = 256, 800,000 of 1, 150 / 229, and 500,000 0.82 times.  With n = 1 merge
+// is the SpMV kernel, the hybrid one lane per row: 1M power law, 124 / 94.
 int spmm_auto_gb300_alg(int m, long long nnz, long long max_row_len, int n, int b_type) {
     const int a = spmm_select_alg_gb300(m, nnz, max_row_len, n, b_type);
     if (a != SPMM_ALG_ROW_SPLIT_HYBRID) return a;
-    const long long row_bytes = (long long)n * (dtype_size(b_type) ? dtype_size(b_type) : 4);
+    const int elem = dtype_size(b_type) ? dtype_size(b_type) : 4;
+    const long long row_bytes = (long long)n * elem;
     const bool type1 = max_row_len > 1024 && max_row_len * 8192 >= nnz;
-    const bool ahead = n > 1 && row_bytes % 16 == 0 &&
-                       (type1 ? row_bytes <= 64 && nnz >= (8LL << 20) : row_bytes <= 256 && nnz >= 1500000);
+    const bool shortest = nnz * 4 < m * 9LL;  // below 2.25 nonzeros per row
+    bool ahead = false;
+    if (row_bytes % 16 != 0) ahead = type1 && n == 2 && nnz >= 12000000;
+    else if (type1) ahead = row_bytes <= 64 ? nnz >= 6000000 : elem == 2 && nnz >= 4000000;
+    else if (row_bytes <= 128) ahead = nnz >= (shortest ? 1000000 : 1500000);
+    else if (row_bytes <= 256 && elem == 2) ahead = shortest || nnz >= 300000;
+    else if (row_bytes <= 256) ahead = nnz >= (!shortest ? 1500000 : row_bytes < 256 ? 450000 : 1100000);
+    else if (row_bytes >= 512) ahead = m >= 520000 && (elem == 4 || row_bytes < 640);
     return ahead ? a : (int)SPMM_ALG_MERGE;
 }
 

@@ -50,3 +50,22 @@ def test_a_workspace_for_the_selected_family_is_enough(gpu_lib, n):
     with pytest.raises(gpu_lib.SpMMError) as e:
         gpu_lib.spmm(rp, ci, v, B, alg="auto_gb300", nnz=nnz, tuning=hint, workspace=ws[:1024])
     assert e.value.status == gpu_lib.ERR_WORKSPACE
+
+
+def test_the_hybrid_stays_where_it_is_ahead():
+    """Both sides of the lines, at sizes where both families were timed."""
+    pkg.build()
+    F, H, M = pkg.F32, pkg.BF16, 1_000_000
+    hybrid = [(400_000, 11_120_000, 40_000, 64, H), (200_000, 5_260_000, 20_000, 40, H), (300_000, 6_690_000, 30_000, 8, F),
+              (M, 23_500_000, 100_000, 2, F), (500_000, 500_000, 1, 128, H), (50_000, 50_000, 1, 96, H),
+              (800_000, 800_000, 1, 256, H), (1_200_000, 1_200_000, 1, 40, F), (500_000, M, 2, 48, F),
+              (1_200_000, 2_400_000, 2, 128, F), (1_200_000, 2_400_000, 2, 192, F), (1_200_000, 1_200_000, 1, 64, F),
+              (800_000, 1_600_000, 2, 32, F)]
+    merge = [(100_000, 1_900_000, 10_000, 64, H), (200_000, 5_260_000, 20_000, 16, H), (200_000, 5_260_000, 20_000, 16, F),
+             (M, 23_500_000, 100_000, 32, F), (M, 23_500_000, 100_000, 5, F), (M, 23_500_000, 100_000, 1, F),
+             (500_000, 500_000, 1, 256, H), (800_000, 800_000, 1, 160, H), (M, 2 * M, 2, 100, H), (200_000, 200_000, 1, 48, F),
+             (500_000, 500_000, 1, 128, F), (M, 2 * M, 2, 100, F), (800_000, 800_000, 1, 32, F)]
+    for alg, cases in ((pkg.ALG_ROW_SPLIT_HYBRID, hybrid), (pkg.ALG_MERGE, merge)):
+        for c in cases:
+            assert pkg.spmm_select_alg_gb300(*c) == pkg.ALG_ROW_SPLIT_HYBRID, c
+            assert pkg.spmm_auto_gb300_alg(*c) == alg, c
