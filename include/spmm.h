@@ -202,12 +202,14 @@ double spmm_tiled_reuse(int m, int k, long long nnz, int n, int b_type);
 /*
  * Column slabs the library uses by default for a product of algorithm alg
  * (a spmm_alg_t after selection) with k rows of B and n columns of b_type on
- * the current device.  Row split: where half of the device's L2 does not hold
+ * the current device, where A has k rows of 8 nonzeros.  Row split: where half of the device's L2 does not hold
  * the 512 bytes per row of B that a pass covers, one per 256 bytes if it holds
  * these, else one per 128, for rows of 256 bytes or more that the slabs exceed
  * by at most a seventh (semirings other than (+, x): 512 bytes or more).
  * Otherwise 2 when B is larger than twice the L2 and its rows are wide (>= 512
- * bytes for merge, >= 256 bytes otherwise), else 1.
+ * bytes for merge, >= 256 bytes otherwise), else 1.  Products of longer rows or
+ * of fewer nonzeros per row of B, which narrow slabs do not repay, take the
+ * latter number in the place of the former where the slabs are many.
  * Each slab pass gathers that share of every row of B from a B slab that
  * much smaller.  Reads the L2 size of the current device (no device work).
  * Products whose B and C are not 16-byte aligned take more slabs where a pass

@@ -177,25 +177,53 @@ bool hybrid_two_vectors(int n, int b_type, long long ldb, long long ldc, const S
     return b_type == SPMM_F32 && s.vec == 4 && n >= 32 && n % 8 == 0 && ldb % 8 == 0 && ldc % 8 == 0;
 }
 
+// Whether row split slabs of `width` bytes of a row (`pieces` of them) are faster
+// than its wide passes over the same columns.  Every pass walks A again, the
+// longer the rows the longer; what it saves are gathers that miss L2.  So it has
+// to be repaid by slabs that L2 holds, by enough nonzeros on a row of B to find it
+// there again (float32, whose wide passes are bound by the gathers alone) or by
+// lanes that the wide passes leave idle.  Measured on GB300 over k = 150,000 to
+// 2.5M, wide passes = 1: float32, 400,000 rows of B, 8 nonzeros on each, rows of
+// A of 8 / 32 / 100: 4 pieces 0.81 / 0.72 / 0.81, 6 (wide ones leave a quarter of
+// the lanes idle) 0.74 / 0.85 / 0.92, 8 pieces 0.91 / 1.05 / 1.07, 16 pieces 1.10
+// / 1.36 / 1.35; 900,000 rows of B: 3 pieces 0.82 / 0.87 / 0.90, 4 0.97 / 1.04 /
+// 1.08, 6 0.85 / 1.00 / 1.05; 2M rows with one nonzero each, 4 pieces 1.06; bf16,
+// 900,000 rows: 4 pieces 0.86 / 0.95 / 1.01, 8 0.88 / 0.94 / 1.02, 16 0.94 / 1.03
+// / 1.14.
+bool narrow_slabs_pay(long long pieces, long long width, double lanes_used, int m, int k, long long nnz, int elem,
+                      long long l2) {
+    const double d = (double)nnz / m, slab = (double)k * width / l2;
+    const bool idle = lanes_used <= 0.875, rare = nnz < 4LL * k;
+    // long rows, too few of them to fill the GPU with more passes
+    if (d >= 64 && rare && m * pieces < (elem == 2 ? 20000 : 40000) && !(idle && elem == 2)) return false;
+    if (width > 128) return pieces <= 8 || d < 16 || elem == 2 || slab > 0.4;
+    const bool fits = slab <= 2.0 / 3;
+    if (elem == 2)
+        return pieces <= 2 || d < 16 || (pieces <= 16 && d < 24) || (pieces <= 10 && idle) ||
+               (pieces <= (d < 64 ? 12 : 8) && slab <= 2 && (fits || d < 64));
+    if (idle && pieces <= 10)
+        return lanes_used <= 0.65 || fits || d < 24 || (pieces <= 3 && (d < 64 || !rare));
+    if (nnz < 2LL * k) return false;
+    return pieces <= 2 || (pieces <= 4 && (d < 64 ? fits : slab <= 0.5)) || (pieces <= 8 && d < 16 && slab <= 1);
+}
+
 // Column slabs: each pass gathers a part of every row, over a B slab that much
 // smaller and so more likely to be found in L2.
 //
 // Row split: a pass covers 512 bytes of a row (32 lanes).  Where half of L2 does
 // not hold that much of B, slabs of 256 or 128 bytes do (128 if neither does),
 // for rows of 256 bytes or more (512 for the semirings, whose walk costs more)
-// that leave at most a seventh of the last pass to spare.  A pass costs another
-// read of A and another walk, which is repaid as soon as the gathers miss.
-// Measured on GB300, one pass (above 2 L2: two) against these: bf16 n = 128, 1M
-// rows of 32, 0.99 -> 0.81 ms; float32 n = 128, 500,000 of 32, 0.93 -> 0.59; 1M
-// of 16, 0.96 -> 0.90; n = 256, 500,000 of 32, 1.86 -> 1.18; n = 64, 500,000 of
-// 32, 0.36 -> 0.29; B of 82 MB, n = 128, 0.209 -> 0.192 ms.  Where 512 bytes fit,
-// 128 cost (n = 256, 200,000 rows of 37, k = 85,000: 0.37 -> 0.41 ms), and so do four passes for the
-// 3.1 of n = 100 (0.264 -> 0.291 ms).
+// that leave at most a seventh of the last pass to spare (n = 100, 3.1 passes:
+// 0.264 -> 0.291 ms), where narrow_slabs_pay says so.  One pass (above 2 L2: two)
+// against these, ms: bf16 n = 128, 1M rows of 32, 0.99 -> 0.81; float32 n = 128,
+// 500,000 of 32, 0.93 -> 0.59; n = 64, 500,000 of 32, 0.36 -> 0.29; B of 82 MB,
+// n = 128, 0.209 -> 0.192.  Where 512 bytes fit, 128 cost (n = 256, 200,000 rows
+// of 37, k = 85,000: 0.37 -> 0.41).
 //
 // Otherwise 2 when B is larger than twice L2 and its rows are wide (merge with
 // 512-byte rows, the hybrid and ragged row splits from 256 bytes gain 6-14 %;
 // narrower rows lose).
-int default_slabs(int alg, int k, int n, int b_type, bool plus_times) {
+int default_slabs(int alg, int m, int k, long long nnz, int n, int b_type, bool plus_times) {
     static std::atomic<int> l2_cache[64];  // 0 until first queried; every thread stores the same value
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
@@ -204,18 +232,23 @@ int default_slabs(int alg, int k, int n, int b_type, bool plus_times) {
         if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev) != cudaSuccess) return 1;
         l2_cache[dev].store(l2, std::memory_order_relaxed);
     }
-    const long long row_bytes = (long long)n * dtype_size(b_type);
+    const int elem = dtype_size(b_type);
+    const long long row_bytes = (long long)n * elem;
+    const long long min_row = alg == SPMM_ALG_MERGE ? 512 : 256;
+    const int wide = (long long)k * row_bytes > 2LL * l2 && row_bytes >= min_row ? 2 : 1;
     if (alg == SPMM_ALG_ROW_SPLIT && row_bytes >= (plus_times ? 256 : 512) &&
         (long long)k * std::min(row_bytes, 512LL) > l2 / 2) {
+        const long long vecs = (row_bytes + 15) / 16, lanes = pow2_ceil((vecs + wide - 1) / wide);
+        const double used = (double)vecs / ((vecs + lanes - 1) / lanes * lanes);  // of the wide passes' lanes
         const long long width = (long long)k * 256 <= l2 / 2 ? 256 : 128;
         for (long long w = width; w >= 128; w /= 2) {
             const long long pieces = (row_bytes + w - 1) / w;
-            if (pieces * w * 7 <= row_bytes * 8) return (int)std::min<long long>(pieces, 65535);
+            if (pieces * w * 7 > row_bytes * 8) continue;
+            if (!narrow_slabs_pay(pieces, w, used, m, k, nnz, elem, l2)) break;
+            return (int)std::min<long long>(pieces, 65535);
         }
     }
-    if ((long long)k * row_bytes <= 2LL * l2) return 1;
-    const long long min_row = alg == SPMM_ALG_MERGE ? 512 : 256;
-    return row_bytes >= min_row ? 2 : 1;
+    return wide;
 }
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -652,7 +685,7 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
     }
     const int a = resolve_alg(alg, m, nnz, tuning);
     spmm_tuning_t t_eff = tuning ? *tuning : spmm_tuning_t{};
-    if (t_eff.column_slabs <= 0 && t_eff.lanes_per_row <= 0) t_eff.column_slabs = default_slabs(a, k, n, b_type, L->plus_times);
+    if (t_eff.column_slabs <= 0 && t_eff.lanes_per_row <= 0) t_eff.column_slabs = default_slabs(a, m, k, nnz, n, b_type, L->plus_times);
     if (!choose_shape(n, b_type, c_type, B, ldb, C, ldc, &t_eff, &shape)) return SPMM_ERR_INVALID_VALUE;
     if (a == SPMM_ALG_ROW_SPLIT_HYBRID && hybrid_two_vectors(n, b_type, ldb, ldc, shape) && !shape_for(n, 8, &t_eff, &shape))
         return SPMM_ERR_INVALID_VALUE;
@@ -867,7 +900,7 @@ double spmm_tiled_reuse(int m, int k, long long nnz, int n, int b_type) {
 
 int spmm_default_column_slabs(int alg, int k, int n, int b_type) {
     if (k < 0 || n < 0 || dtype_size(b_type) == 0) return 1;
-    return spmm::default_slabs(alg, k, n, b_type, true);
+    return spmm::default_slabs(alg, k, k, 8LL * k, n, b_type, true);  // k rows of 8
 }
 
 int spmm_csr_max_row_length(int m, const int* row_ptr, long long* max_row_len, void* stream) {
