@@ -222,7 +222,10 @@ bool narrow_slabs_pay(long long pieces, long long width, double lanes_used, int 
 //
 // Otherwise 2 when B is larger than twice L2 and its rows are wide (merge with
 // 512-byte rows, the hybrid and ragged row splits from 256 bytes gain 6-14 %;
-// narrower rows lose).
+// narrower rows lose).  Merge rows of 512 bytes stay whole below 3 nonzeros per
+// row of A, where half-rows pay for another walk and for the sum over two lane
+// groups at every row end: 900,000 rows of 1, bf16 n = 256, 265 -> 165 us; of
+// Poisson 1.3, float32 n = 128, 194 -> 181.
 int default_slabs(int alg, int m, int k, long long nnz, int n, int b_type, bool plus_times) {
     static std::atomic<int> l2_cache[64];  // 0 until first queried; every thread stores the same value
     int dev = 0;
@@ -235,7 +238,8 @@ int default_slabs(int alg, int m, int k, long long nnz, int n, int b_type, bool 
     const int elem = dtype_size(b_type);
     const long long row_bytes = (long long)n * elem;
     const long long min_row = alg == SPMM_ALG_MERGE ? 512 : 256;
-    const int wide = (long long)k * row_bytes > 2LL * l2 && row_bytes >= min_row ? 2 : 1;
+    int wide = (long long)k * row_bytes > 2LL * l2 && row_bytes >= min_row ? 2 : 1;
+    if (alg == SPMM_ALG_MERGE && row_bytes <= 512 && nnz < 3LL * m) wide = 1;
     if (alg == SPMM_ALG_ROW_SPLIT && row_bytes >= (plus_times ? 256 : 512) &&
         (long long)k * std::min(row_bytes, 512LL) > l2 / 2) {
         const long long vecs = (row_bytes + 15) / 16, lanes = pow2_ceil((vecs + wide - 1) / wide);
