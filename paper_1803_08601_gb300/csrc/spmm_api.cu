@@ -289,13 +289,15 @@ MergeLayout merge_layout(long long num_tiles, int warps, int n) {
 // tile together) for column slabs of shape s.  With W lanes per row the warp
 // adds up 32 / W lane groups' partial sums at every row end, which short rows
 // do not repay: up to 4 lanes of 16 bytes, 8 lanes below a mean of 4 nonzeros
-// per row and unaligned rows of up to 4 columns below 8 run the narrow kernel.
+// per row, and unaligned rows of up to 4 columns below 8 and of up to 8 below
+// 3.5 run the narrow kernel.
 // Measured on GB300, narrow / the other (us): 300,000 rows of Poisson 8,
 // n = 16, 41 / 51; 400,000 of Poisson 2.5, n = 32, 42 / 46; 700,000 of Poisson
-// 5, n = 32, 94 / 88; 700,000 of Poisson 5, n = 2, 43 / 55.
+// 5, n = 32, 94 / 88; 700,000 of Poisson 5, n = 2, 43 / 55;
+// 500,000 of Poisson 3, n = 5, 48 / 57, 1M of Poisson 4, 93 / 91.
 bool merge_narrow(int m, long long nnz, const Shape& s) {
     if (s.vec > 1) return s.W <= 4 || (s.W == 8 && nnz < 4LL * m);
-    return s.W <= 4 && nnz < 8LL * m;
+    return s.W <= 4 ? nnz < 8LL * m : s.W == 8 && 2 * nnz < 7LL * m;
 }
 
 // Lane layout where 16-byte accesses are not aligned (base.vec == 1): up to 128

@@ -85,3 +85,20 @@ def test_noalloc_keeps_accepting_wide_products(gpu_lib):
                                   None, torch.cuda.current_stream().cuda_stream)
     assert st == gpu_lib.OK, gpu_lib.spmm_status_string(st)
     assert torch.equal(C, gpu_lib.spmm(d_rp, d_ci, d_v, B, alg="row_split", nnz=int(rp[-1])))
+
+
+@pytest.mark.parametrize("n", [5, 6, 7])
+@pytest.mark.parametrize("mean", [1, 3, 4])
+def test_unaligned_short_rows_are_bitwise(gpu_lib, n, mean):
+    """Both sides of the mean row length at which rows of up to 8 unaligned columns change their kernel."""
+    import torch
+
+    rng = np.random.default_rng(10 * n + mean)
+    rp, ci, v = csr_arrays(np.concatenate([rng.poisson(mean, 20_000), np.zeros(70), [900], np.zeros(3)]).astype(np.int64),
+                           5000, 6, int_vals=True)
+    B = rng.integers(-4, 5, size=(5000, n)).astype(np.float32)
+    ref = oracle.spmm(rp, ci, v, B).astype(np.float32)
+    d_rp, d_ci, d_v, d_B = (torch.from_numpy(x).cuda() for x in (rp, ci, v, B))
+    for tuning in (None, dict(column_slabs=2), dict(items_per_subwarp=5)):
+        C = gpu_lib.spmm(d_rp, d_ci, d_v, d_B, alg="merge", nnz=int(rp[-1]), tuning=tuning)
+        assert np.array_equal(C.cpu().numpy(), ref), tuning
