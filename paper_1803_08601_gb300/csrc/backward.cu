@@ -336,6 +336,7 @@ struct SddmmArgs {
     long long ldb;
     void* out;
     int chunk;  // nonzeros per lane group
+    int k;
 };
 
 // One lane group of W lanes per run of `chunk` consecutive nonzeros; each lane
@@ -444,7 +445,8 @@ __global__ void __launch_bounds__(128, sddmm_min_blocks<VEC, E>()) sddmm_warp_ke
     bool col_ok[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) col_ok[e] = col0 + (e * 32 + lane) * VEC < a.n;
-    const int my_col = col_ok[0] ? col0 + lane * VEC : 0;  // lanes past n read along with column 0 and add nothing
+    // lanes past n read along with the pass's first column, which the warp reads anyway, and add nothing
+    const int my_col = col_ok[0] ? col0 + lane * VEC : col0;
     const TD* const b_col = static_cast<const TD*>(a.B) + my_col;
     const TD* const d_col = static_cast<const TD*>(a.dC) + my_col;
     const unsigned ldb_bytes = (unsigned)(a.ldb * (long long)sizeof(TD));
@@ -583,11 +585,31 @@ cudaError_t sddmm_warp_launch(const SddmmArgs& a0, cudaStream_t st) {
     a.chunk = (int)std::max<long long>(32, (per_warp + 31) / 32 * 32);
     const long long blocks = (a.nnz + 4LL * a.chunk - 1) / (4LL * a.chunk);
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    for (int c = 0; c < a.n; c += 32 * VEC * E) {
-        sddmm_warp_kernel<TD, TO, VEC, E><<<(unsigned)blocks, 128, 0, st>>>(a, c, c > 0);
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
+    long long c = 0;
+    auto pass = [&](auto chunks) {
+        constexpr int EP = decltype(chunks)::value;
+        sddmm_warp_kernel<TD, TO, VEC, EP><<<(unsigned)blocks, 128, 0, st>>>(a, (int)c, c > 0);
         if (c > 0) g_launches.fetch_add(1, std::memory_order_relaxed);  // the caller counts one
+        c += 32 * VEC * EP;
+        return cudaGetLastError();
+    };
+    while (c < a.n) {
+        cudaError_t e;
+        const long long left = a.n - c;
+        if constexpr (sizeof(TD) == 4 && VEC == 4 && E == 1) {
+            // A short last pass costs nearly a full one, and joins the pass before it: up to 52 columns,
+            // and any short one where L2 (129 MB) does not hold a pass's columns of B.  Against two passes
+            // and against one with the products reduced one by one (us): 500,000 rows of Poisson 6,
+            // n = 132, 310 / 421 / 363, n = 200, 412 / 490 / 457, n = 256, 488 / 463 / 519; 150,000 of
+            // 15, n = 132, 169 / 199 / 199, n = 200, 236 / 222 / 224.
+            if (left > 128 && left < 256 && (left <= 180 || a.k * 512LL > (129LL << 20)))
+                e = pass(std::integral_constant<int, 2>());
+            else
+                e = pass(std::integral_constant<int, 1>());
+        } else {
+            e = pass(std::integral_constant<int, E>());
+        }
+        if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
@@ -756,7 +778,7 @@ int sddmm_csr(int m, int k, int n, long long nnz, const int* row_ptr, const int*
     if (n > 0 && (!dC || !B || lddc < n || ldb < n)) return SPMM_ERR_INVALID_VALUE;
     if (dc_type != b_type) return SPMM_ERR_UNSUPPORTED;
     if (ldb * (b_type == SPMM_F32 ? 4LL : 2LL) > 0xffffffffLL) return SPMM_ERR_INVALID_VALUE;  // rows of B < 4 GiB apart
-    SddmmArgs a{m, n, nnz, row_ptr, col_ind, dC, lddc, B, ldb, out, 32};
+    SddmmArgs a{m, n, nnz, row_ptr, col_ind, dC, lddc, B, ldb, out, 32, k};
     cudaStream_t s = (cudaStream_t)stream;
     if (n == 0) {  // empty dot products
         const int es = out_type == SPMM_F32 ? 4 : 2;

@@ -44,3 +44,20 @@ def test_strides(gpu_lib, n, pad):
     out = gpu_lib.sddmm(d_rp, d_ci, d_dC[:, :n], d_B[:, :n])
     ref = oracle.sddmm(rp, ci, np.ascontiguousarray(dC[:, :n]), np.ascontiguousarray(B[:, :n]))
     assert np.array_equal(out.cpu().numpy(), ref.astype(np.float32))
+
+
+@pytest.mark.parametrize("n", [132, 180, 184, 252, 260, 388])
+@pytest.mark.parametrize("k", [7000, 300_000])
+def test_last_passes_are_bitwise(gpu_lib, n, k):
+    """Widths whose last pass joins the one before it, always or where B is large."""
+    import torch
+
+    rng = np.random.default_rng(n)
+    rp, ci, _ = csr_arrays(np.concatenate([rng.integers(0, 9, 600), [0, 300, 0, 31, 33]]).astype(np.int64), k, 9)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    dC = rng.integers(-3, 4, size=(len(rp) - 1, n)).astype(np.float32)
+    B = torch.randint(-4, 5, (k, n), device="cuda", generator=g).float()
+    d_rp, d_ci, d_dC = (torch.from_numpy(x).cuda() for x in (rp, ci, dC))
+    out = gpu_lib.sddmm(d_rp, d_ci, d_dC, B)
+    rows = torch.repeat_interleave(torch.arange(len(rp) - 1, device="cuda"), (d_rp[1:] - d_rp[:-1]).long())
+    assert torch.equal(out, (d_dC[rows] * B[d_ci.long()]).sum(1))
