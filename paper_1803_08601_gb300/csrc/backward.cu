@@ -645,15 +645,23 @@ int sddmm_run(const SddmmArgs& a0, cudaStream_t st) {
     // A warp per nonzero, with the narrowest access that covers the row in one pass of 32 lanes, or
     // the widest aligned one and several passes (float32 results) or column chunks (16-bit results,
     // which cannot be added up in place).  The lane groups stay for up to 3 columns and, up to 32
-    // aligned ones (or 8), for rows of A of fewer than 4 nonzeros, where the warp changes rows at
-    // every other nonzero: 600,000 rows of 3, n = 32, 119 us against 129; 2M nonzeros of a graph,
-    // n = 32, 80 against 64; 900,000 of Poisson 15, n = 8, 72 against 31.
+    // aligned ones (or 8), for rows of A of fewer than 4 nonzeros (4.75 for up to 7 unaligned columns),
+    // where the warp changes rows at every other nonzero: 600,000 rows of 3, n = 32, 119 us against
+    // 129; 2M nonzeros of a graph, n = 32, 80 against 64; 900,000 of Poisson 15, n = 8, 72 against 31.
+    // They also stay for rows of up to 4 lanes where many nonzeros fill their waves (of 4 CTAs per SM,
+    // about as long as they are empty), the groups / the warps (us): n = 16, 500,000 rows of 9.5, 120 /
+    // 146, of 6, 115 / 119, 800,000 of 7 (1.1 waves) 228 / 197; n = 8, 1M of 6, 154 / 187, bf16 n = 16,
+    // 1M of 9, 175 / 238; bf16 n = 4 (unaligned), 500,000 of 8, 97 / 120, of 4.5, 87 / 89.
     constexpr bool kPasses = sizeof(TO) == 4;
     const int n = a.n;
     int w = V;
     while (w > 1 && !aligned(w)) w >>= 1;
-    const bool by_groups = n < 4 || (n <= 32 && a.nnz < 4LL * a.m && (n <= 8 || vec_ok)) ||
-                        (!kPasses && n > (w == V ? 256 * V : 128));
+    const bool short_rows = n <= 32 && (n < 8 && !vec_ok ? 4 * a.nnz < 19LL * a.m : a.nnz < 4LL * a.m) && (n <= 8 || vec_ok);
+    const long long wave = 4LL * 152 * (kThreads / W) * 128;  // nonzeros of the lane groups' CTAs
+    const bool full = vec_ok ? W <= 4 && a.nnz >= (W > 1 || kPasses ? 3600000 : 7000000) &&
+                                   (a.nnz <= wave || a.nnz * 100 >= (a.nnz + wave - 1) / wave * wave * 69)
+                             : n == 4 && a.nnz >= 2500000;
+    const bool by_groups = n < 4 || short_rows || full || (!kPasses && n > (w == V ? 256 * V : 128));
     if (!by_groups) {
         if (n <= 32) return launched(sddmm_warp_launch<TD, TO, 1, 1>(a, st));
         if (w >= 2 && n <= 64) return launched(sddmm_warp_launch<TD, TO, 2, 1>(a, st));

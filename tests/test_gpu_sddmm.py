@@ -61,3 +61,19 @@ def test_last_passes_are_bitwise(gpu_lib, n, k):
     out = gpu_lib.sddmm(d_rp, d_ci, d_dC, B)
     rows = torch.repeat_interleave(torch.arange(len(rp) - 1, device="cuda"), (d_rp[1:] - d_rp[:-1]).long())
     assert torch.equal(out, (d_dC[rows] * B[d_ci.long()]).sum(1))
+
+
+@pytest.mark.parametrize("n,storage,nnz", [(16, "float32", 3_600_000), (16, "float32", 3_599_999), (4, "bfloat16", 2_500_000),
+                                           (8, "bfloat16", 7_000_000), (5, "float32", 185_000), (5, "float32", 195_000)])
+def test_the_lines_between_lane_groups_and_warps(gpu_lib, n, storage, nnz):
+    import torch
+
+    g = torch.Generator(device="cuda").manual_seed(nnz)
+    m, k, dt = 40_000, 5000, getattr(torch, storage)
+    rp = (torch.arange(m + 1, device="cuda", dtype=torch.int64) * nnz // m).int()
+    ci = torch.randint(k, (nnz,), device="cuda", generator=g).int()
+    dC = torch.randint(-3, 4, (m, n), device="cuda", generator=g).to(dt)
+    B = torch.randint(-4, 5, (k, n), device="cuda", generator=g).to(dt)
+    rows = torch.repeat_interleave(torch.arange(m, device="cuda"), (rp[1:] - rp[:-1]).long())
+    out = gpu_lib.sddmm(rp, ci, dC, B)
+    assert torch.equal(out, (dC[rows].float() * B[ci.long()].float()).sum(1).to(dt))
