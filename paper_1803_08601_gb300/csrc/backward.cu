@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(128, sddmm_min_blocks<VEC, E>()) sddmm_warp_ke
     int* const w_col = s_col[warp];
     bool col_ok[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) col_ok[e] = col0 + (e * 32 + lane) * VEC < a.n;
+    for (int e = 0; e < E; ++e) col_ok[e] = (e * 32 + lane) * VEC < a.n - col0;  // a.n may be near 2^31
     // lanes past n read along with the pass's first column, which the warp reads anyway, and add nothing
     const int my_col = col_ok[0] ? col0 + lane * VEC : col0;
     const TD* const b_col = static_cast<const TD*>(a.B) + my_col;
