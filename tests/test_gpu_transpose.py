@@ -25,3 +25,38 @@ def test_tile_and_digit_edges(gpu_lib, nnz, k):
     ref = oracle.csr_transpose(rp, ci, k)
     for got, want in zip((rpt, cit, perm), ref):
         assert np.array_equal(got.cpu().numpy(), want)
+
+
+def sparse_rows(gap, m=300_000):
+    """Nonzeros in the first and the last few rows and `gap` empty rows between two of one tile."""
+    lens = np.concatenate([np.full(900, 3), np.zeros(gap), [1, 0, 4], np.zeros(m - 1003), np.full(100, 20)])
+    return np.concatenate([[0], np.cumsum(lens)]).astype(np.int32)
+
+
+@pytest.mark.parametrize("gap", [4000, 8100, 8192, 8193, 3_000_000])
+def test_long_runs_of_empty_rows(gpu_lib, gap):
+    import torch
+
+    rp = sparse_rows(gap)
+    ci = np.random.default_rng(gap).integers(0, 5000, rp[-1]).astype(np.int32)
+    got = gpu_lib.csr_transpose(*(torch.from_numpy(x).cuda() for x in (rp, ci)), 5000)
+    for x, want in zip(got, oracle.csr_transpose(rp, ci, 5000)):
+        assert np.array_equal(x.cpu().numpy(), want)
+
+
+def test_work_does_not_grow_with_the_empty_rows(gpu_lib):
+    """20M empty rows between two nonzeros: the few kernels of a transpose take well below a millisecond, one CTA's
+    walk over the rows tens of them."""
+    import torch
+
+    rp = torch.from_numpy(sparse_rows(20_000_000)).cuda()
+    ci = torch.randint(5000, (int(rp[-1]),), device="cuda").int()
+    times = []
+    for _ in range(5):
+        t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t0.record()
+        gpu_lib.csr_transpose(rp, ci, 5000)
+        t1.record()
+        t1.synchronize()
+        times.append(t0.elapsed_time(t1))
+    assert min(times) < 5.0, times
