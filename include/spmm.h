@@ -228,6 +228,14 @@ int spmm_default_column_slabs(int alg, int k, int n, int b_type);
 int spmm_csr_max_row_length(int m, const int *row_ptr, long long *max_row_len, void *stream);
 
 /*
+ * The same for a row_ptr that is still being written: the row lengths are read
+ * behind `event` (a cudaEvent_t, recorded after the work that writes row_ptr), on
+ * a stream of the library's own, so that the call waits for that work and not for
+ * what the caller has queued behind it.
+ */
+int spmm_csr_max_row_length_after(int m, const int *row_ptr, long long *max_row_len, void *event);
+
+/*
  * C = A B in float32 (vals, B, C all float32), the signature of the paper's
  * problem statement (Section 1).  alg is a spmm_alg_t.  For SPMM_ALG_AUTO the
  * heuristic needs nnz = row_ptr[m], which this call reads back from the device

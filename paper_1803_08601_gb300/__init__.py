@@ -67,6 +67,7 @@ _SIGNATURES = {
     "spmm_default_column_slabs": ([_i, _i, _i, _i], _i),
     "spmm_tiled_reuse": ([_i, _i, _ll, _i, _i], _d),
     "spmm_csr_max_row_length": ([_i, _vp, ctypes.POINTER(_ll), _vp], _i),
+    "spmm_csr_max_row_length_after": ([_i, _vp, ctypes.POINTER(_ll), _vp], _i),
     "spmm_csr": ([_i, _i, _i, _vp, _vp, _vp, _vp, _ll, _vp, _ll, _i, _vp], _i),
     "spmm_csr_ex": ([_i, _i, _i, _ll, _vp, _vp, _vp, _i, _vp, _i, _ll, _vp, _i, _ll, _i, _TP, _vp, _sz, _vp, _vp], _i),
     "spmm_csr_semiring": ([_i, _i, _i, _ll, _vp, _vp, _vp, _vp, _ll, _vp, _ll, _i, _i, _TP, _vp, _sz, _vp, _vp], _i),
@@ -153,6 +154,13 @@ def spmm_csr_max_row_length(m, row_ptr, stream) -> tuple[int, int]:
     return st, out.value
 
 
+def spmm_csr_max_row_length_after(m, row_ptr, event) -> tuple[int, int]:
+    """Returns (status, longest row)."""
+    out = ctypes.c_longlong(0)
+    st = load().spmm_csr_max_row_length_after(m, row_ptr, ctypes.byref(out), event)
+    return st, out.value
+
+
 def default_column_slabs(alg: int, k: int, n: int, b_type: int = F32) -> int:
     return load().spmm_default_column_slabs(alg, k, n, b_type)
 
@@ -166,8 +174,14 @@ def gather_probe(B, idx, row_bytes: int, out, stream=None) -> None:
                                     out.data_ptr(), _stream_handle(stream)), "spmm_gather_probe")
 
 
-def max_row_length(row_ptr, stream=None) -> int:
+def max_row_length(row_ptr, stream=None, after=None) -> int:
+    """The longest row; with ``after``, an event recorded behind the work that writes row_ptr, read as soon as that
+    is done, whatever is queued behind it."""
     _require_cuda(row_ptr)
+    if after is not None:
+        st, v = spmm_csr_max_row_length_after(row_ptr.numel() - 1, row_ptr.data_ptr(), int(after.cuda_event))
+        _check(st, "spmm_csr_max_row_length_after")
+        return v
     st, v = spmm_csr_max_row_length(row_ptr.numel() - 1, row_ptr.data_ptr(), _stream_handle(stream))
     _check(st, "spmm_csr_max_row_length")
     return v

@@ -36,21 +36,23 @@ class CSRMatrix:
         Work queued on the stream before transpose_pattern() is called overlaps that call's wait."""
         if self._t is None and self._t_queued is None:
             parts = csr_transpose(self.row_ptr, self.col_ind, self.k)
-            probe = torch.cuda.Stream()
-            probe.wait_stream(torch.cuda.current_stream())
-            self._t_queued = (*parts, probe)
+            done = torch.cuda.Event()
+            done.record()
+            self._t_queued = parts, done
 
     def transpose_pattern(self):
         """(row_ptr_t, col_ind_t, perm, max_row_t) of A^T, built on first use."""
         t, queued = self._t, self._t_queued
         if t is None:
             if queued is None:
-                parts = csr_transpose(self.row_ptr, self.col_ind, self.k)
-                t = (*parts, max_row_length(parts[0]))
+                    parts = csr_transpose(self.row_ptr, self.col_ind, self.k)
+                longest = max_row_length(parts[0])
             else:
-                # the longest row is read on a stream of its own, which waits for the transpose only; the call
-                # returns once that stream is done, so the parts are complete for every stream from here on
-                t = (*queued[:3], max_row_length(queued[0], stream=queued[3]))
+                # the longest row is read behind the transpose, not behind what was queued after it; the call
+                # returns once it is known, so the parts are complete for every stream from here on
+                parts, done = queued
+                longest = max_row_length(parts[0], after=done)
+            t = (*parts, longest)
             self._t, self._t_queued = t, None
         return t
 

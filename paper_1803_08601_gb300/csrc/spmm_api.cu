@@ -595,6 +595,19 @@ bool copy_streams(cudaStream_t* up, cudaStream_t* down) {
     return true;
 }
 
+// The stream of spmm_csr_max_row_length_after, one per device, created once: no
+// caller's work is ever queued on it.
+bool probe_stream(cudaStream_t* out) {
+    static std::mutex mu;
+    static cudaStream_t streams[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!streams[dev] && cudaStreamCreateWithFlags(&streams[dev], cudaStreamNonBlocking) != cudaSuccess) return false;
+    *out = streams[dev];
+    return true;
+}
+
 int cuda_status(cudaError_t e) {
     if (e == cudaSuccess) return SPMM_OK;
     if (e == cudaErrorMemoryAllocation) return SPMM_ERR_ALLOC;
@@ -914,6 +927,17 @@ int spmm_csr_max_row_length(int m, const int* row_ptr, long long* max_row_len, v
     *max_row_len = 0;
     if (m == 0) return SPMM_OK;
     return probe_rows(row_ptr, m, (cudaStream_t)stream, max_row_len, nullptr);
+}
+
+int spmm_csr_max_row_length_after(int m, const int* row_ptr, long long* max_row_len, void* event) {
+    if (m < 0 || !max_row_len || !event || (m > 0 && !row_ptr)) return SPMM_ERR_INVALID_VALUE;
+    *max_row_len = 0;
+    cudaStream_t s = nullptr;
+    if (!probe_stream(&s)) return SPMM_ERR_CUDA;
+    const cudaError_t e = cudaStreamWaitEvent(s, (cudaEvent_t)event, 0);
+    if (e != cudaSuccess) return cuda_status(e);
+    if (m == 0) return cuda_status(cudaStreamSynchronize(s));
+    return probe_rows(row_ptr, m, s, max_row_len, nullptr);
 }
 
 size_t spmm_csr_workspace_size(int m, int k, int n, long long nnz, int alg, int b_type, const spmm_tuning_t* tuning) {

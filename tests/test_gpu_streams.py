@@ -49,3 +49,21 @@ def test_queued_on_one_stream_used_on_another(gpu_lib):
     torch.cuda.synchronize()
     assert np.array_equal(dB.cpu().numpy(), ref_dB)
     assert A.transpose_pattern()[3] == int(torch.bincount(ci.long(), minlength=3000).max())
+
+
+def test_the_probe_takes_no_stream_of_torchs_pool(gpu_lib, monkeypatch):
+    """torch hands the 32 streams of its pool out in turn: one taken here would be some caller's as well."""
+    import torch
+
+    (rp, ci, _, _, _), _ = problem(torch, gpu_lib)
+
+    stream = torch.cuda.Stream
+
+    def taken(*args, **kw):  # an object of a stream that is there names its id
+        assert "stream_id" in kw, "a stream of the pool"
+        return stream(*args, **kw)
+
+    A = gpu_lib.CSRMatrix(rp, ci, (4000, 3000))
+    monkeypatch.setattr(torch.cuda, "Stream", taken)
+    A.queue_transpose()
+    assert A.transpose_pattern()[3] == int(torch.bincount(ci.long(), minlength=3000).max())
