@@ -10,7 +10,7 @@ from __future__ import annotations
 
 import torch
 
-from . import ALG_AUTO_GB300, SpmmTuning, csr_transpose, gather_values, max_row_length, sddmm, spmm
+from . import ALG_AUTO_GB300, SpmmTuning, _stream_handle, csr_transpose, gather_values, max_row_length, sddmm, spmm
 
 
 class CSRMatrix:
@@ -24,6 +24,7 @@ class CSRMatrix:
         self._max_row = None
         self._t = None
         self._t_queued = None
+        self._t_home = None
 
     @property
     def max_row(self) -> int:
@@ -35,24 +36,28 @@ class CSRMatrix:
         """Queue the construction of A^T on the current stream, if it is not there yet, without waiting for it.
         Work queued on the stream before transpose_pattern() is called overlaps that call's wait."""
         if self._t is None and self._t_queued is None:
+            home = _stream_handle()
             parts = csr_transpose(self.row_ptr, self.col_ind, self.k)
             done = torch.cuda.Event()
             done.record()
-            self._t_queued = parts, done
+            self._t_queued = parts, done, home
 
     def transpose_pattern(self):
-        """(row_ptr_t, col_ind_t, perm, max_row_t) of A^T, built on first use."""
+        """(row_ptr_t, col_ind_t, perm, max_row_t) of A^T, built on first use.  The tensors belong to the stream that
+        built them: use on another one is recorded with it by spmm_t, and left to the caller elsewhere."""
         t, queued = self._t, self._t_queued
         if t is None:
             if queued is None:
-                    parts = csr_transpose(self.row_ptr, self.col_ind, self.k)
+                home = _stream_handle()
+                parts = csr_transpose(self.row_ptr, self.col_ind, self.k)
                 longest = max_row_length(parts[0])
             else:
                 # the longest row is read behind the transpose, not behind what was queued after it; the call
                 # returns once it is known, so the parts are complete for every stream from here on
-                parts, done = queued
+                parts, done, home = queued
                 longest = max_row_length(parts[0], after=done)
             t = (*parts, longest)
+            self._t_home = home
             self._t, self._t_queued = t, None
         return t
 
@@ -68,6 +73,9 @@ class CSRMatrix:
     def spmm_t(self, vals, dC, alg=ALG_AUTO_GB300):
         """A^T @ dC with vals in A's order (gathered into A^T's order on the device)."""
         rpt, cit, perm, max_row_t = self.transpose_pattern()
+        if _stream_handle() != self._t_home:  # their memory is not given out again before this stream has read them
+            for x in (rpt, cit, perm):
+                x.record_stream(torch.cuda.current_stream())
         vals_t = gather_values(perm, vals)
         return spmm(rpt, cit, vals_t, dC, alg=alg, nnz=self.nnz, tuning={"max_row_len": max_row_t})
 

@@ -51,6 +51,34 @@ def test_queued_on_one_stream_used_on_another(gpu_lib):
     assert A.transpose_pattern()[3] == int(torch.bincount(ci.long(), minlength=3000).max())
 
 
+@pytest.mark.parametrize("queued", [True, False])
+def test_the_transpose_outlives_its_matrix_on_another_stream(gpu_lib, queued):
+    """Memory of A^T, made on one stream, is not given out again while another stream still has to read it, after
+    the last reference is gone.  Nothing is written to what is given out, whoever it belongs to."""
+    import torch
+
+    (rp, ci, v, _, dC), (ref_dB, _) = problem(torch, gpu_lib)
+    A = gpu_lib.CSRMatrix(rp, ci, (4000, 3000))
+    first, second = torch.cuda.Stream(), torch.cuda.Stream()
+    gpu_lib.CSRMatrix(rp, ci, (4000, 3000)).spmm_t(v, dC)  # loads the kernels
+    torch.cuda.synchronize()
+    with torch.cuda.stream(first):
+        if queued:
+            A.queue_transpose()
+        held = [x.untyped_storage().nbytes() for x in A.transpose_pattern()[:3]]
+        taken = {x.data_ptr() for x in A.transpose_pattern()[:3]}
+    with torch.cuda.stream(second):
+        torch.cuda._sleep(200_000_000)  # about a tenth of a second
+        dB = A.spmm_t(v, dC)
+    del A
+    with torch.cuda.stream(first):
+        again = [torch.empty(n, dtype=torch.uint8, device="cuda") for n in held for _ in range(3)]
+    assert not second.query()
+    assert not taken & {x.data_ptr() for x in again}
+    torch.cuda.synchronize()
+    assert np.array_equal(dB.cpu().numpy(), ref_dB)
+
+
 def test_the_probe_takes_no_stream_of_torchs_pool(gpu_lib, monkeypatch):
     """torch hands the 32 streams of its pool out in turn: one taken here would be some caller's as well."""
     import torch
