@@ -355,7 +355,6 @@ struct SddmmArgs {
     long long ldb;
     void* out;
     int chunk;  // nonzeros per lane group
-    int k;
 };
 
 // One lane group of W lanes per run of `chunk` consecutive nonzeros; each lane
@@ -596,7 +595,7 @@ __global__ void __launch_bounds__(128, sddmm_min_blocks<VEC, E>()) sddmm_warp_ke
 }
 
 template <typename TD, typename TO, int VEC, int E>
-cudaError_t sddmm_warp_launch(const SddmmArgs& a0, cudaStream_t st) {
+cudaError_t sddmm_warp_launch(const SddmmArgs& a0, cudaStream_t st, int k = 0) {
     SddmmArgs a = a0;
     // nonzeros per warp: about 256, in whole waves of the 32 warps that an SM runs at once
     const long long wave = 256LL * 32 * 152, waves = std::max<long long>(1, (a.nnz + wave / 2) / wave);
@@ -617,11 +616,13 @@ cudaError_t sddmm_warp_launch(const SddmmArgs& a0, cudaStream_t st) {
         const long long left = a.n - c;
         if constexpr (sizeof(TD) == 4 && VEC == 4 && E == 1) {
             // A short last pass costs nearly a full one, and joins the pass before it: up to 52 columns,
-            // and any short one where L2 (129 MB) does not hold a pass's columns of B.  Against two passes
+            // and any short one where L2 (129 MB) does not hold a pass's columns of B.  Below 5 nonzeros
+            // per row, where every pass loads a row of dC for a few products, passes go two by two.  Against two passes
             // and against one with the products reduced one by one (us): 500,000 rows of Poisson 6,
             // n = 132, 310 / 421 / 363, n = 200, 412 / 490 / 457, n = 256, 488 / 463 / 519; 150,000 of
             // 15, n = 132, 169 / 199 / 199, n = 200, 236 / 222 / 224.
-            if (left > 128 && left < 256 && (left <= 180 || a.k * 512LL > (129LL << 20)))
+            const bool short_rows = a.nnz < 5LL * a.m;
+            if (left > 128 && (short_rows || (left < 256 && (left <= 180 || k * 512LL > (129LL << 20)))))
                 e = pass(std::integral_constant<int, 2>());
             else
                 e = pass(std::integral_constant<int, 1>());
@@ -649,7 +650,7 @@ cudaError_t sddmm_launch_vec(const SddmmArgs& a, int W, long long groups, cudaSt
 }
 
 template <typename TD, typename TO>
-int sddmm_run(const SddmmArgs& a0, cudaStream_t st) {
+int sddmm_run(const SddmmArgs& a0, int k, cudaStream_t st) {
     SddmmArgs a = a0;
     constexpr int V = Elem<TD>::kVec;
     auto aligned = [&](int v) {
@@ -670,16 +671,18 @@ int sddmm_run(const SddmmArgs& a0, cudaStream_t st) {
     // They also stay for rows of up to 4 lanes where many nonzeros fill their waves (of 4 CTAs per SM,
     // about as long as they are empty), the groups / the warps (us): n = 16, 500,000 rows of 9.5, 120 /
     // 146, of 6, 115 / 119, 800,000 of 7 (1.1 waves) 228 / 197; n = 8, 1M of 6, 154 / 187, bf16 n = 16,
-    // 1M of 9, 175 / 238; bf16 n = 4 (unaligned), 500,000 of 8, 97 / 120, of 4.5, 87 / 89.
+    // 1M of 9, 175 / 238; n = 4, 1M of 9, 169 / 234; bf16 n = 4 (unaligned), 500,000 of 8, 97 / 120, of
+    // 4.5, 87 / 89.
     constexpr bool kPasses = sizeof(TO) == 4;
     const int n = a.n;
     int w = V;
     while (w > 1 && !aligned(w)) w >>= 1;
-    const bool short_rows = n <= 32 && (n < 8 && !vec_ok ? 4 * a.nnz < 19LL * a.m : a.nnz < 4LL * a.m) && (n <= 8 || vec_ok);
+    const bool short_rows = n <= 32 && (n < 8 && !vec_ok && a.nnz >= 2000000 ? 4 * a.nnz < 19LL * a.m : a.nnz < 4LL * a.m) && (n <= 8 || vec_ok);
     const long long wave = 4LL * 152 * (kThreads / W) * 128;  // nonzeros of the lane groups' CTAs
-    const bool full = vec_ok ? W <= 4 && a.nnz >= (W > 1 || kPasses ? 3600000 : 7000000) &&
-                                   (a.nnz <= wave || a.nnz * 100 >= (a.nnz + wave - 1) / wave * wave * 69)
-                             : n == 4 && a.nnz >= 2500000;
+    const bool full = !vec_ok   ? n == 4 && a.nnz >= 2500000
+                      : W == 1  ? a.nnz >= 7000000
+                      : W <= 4  ? a.nnz >= 3600000 && (a.nnz <= wave || a.nnz * 100 >= (a.nnz + wave - 1) / wave * wave * (W == 2 ? 69 : 90))
+                                : false;
     const bool by_groups = n < 4 || short_rows || full || (!kPasses && n > (w == V ? 256 * V : 128));
     if (!by_groups) {
         if (n <= 32) return launched(sddmm_warp_launch<TD, TO, 1, 1>(a, st));
@@ -687,7 +690,7 @@ int sddmm_run(const SddmmArgs& a0, cudaStream_t st) {
         if constexpr (V == 8) {
             if (w >= 4 && n <= 128) return launched(sddmm_warp_launch<TD, TO, 4, 1>(a, st));
         }
-        if (w == V && (n <= 32 * V || kPasses)) return launched(sddmm_warp_launch<TD, TO, V, 1>(a, st));
+        if (w == V && (n <= 32 * V || kPasses)) return launched(sddmm_warp_launch<TD, TO, V, 1>(a, st, k));
         if constexpr (!kPasses) {
             if (w == V && n <= 64 * V) return launched(sddmm_warp_launch<TD, TO, V, 2>(a, st));
             if (w == V && n <= 128 * V) return launched(sddmm_warp_launch<TD, TO, V, 4>(a, st));
@@ -805,17 +808,17 @@ int sddmm_csr(int m, int k, int n, long long nnz, const int* row_ptr, const int*
     if (n > 0 && (!dC || !B || lddc < n || ldb < n)) return SPMM_ERR_INVALID_VALUE;
     if (dc_type != b_type) return SPMM_ERR_UNSUPPORTED;
     if (ldb * (b_type == SPMM_F32 ? 4LL : 2LL) > 0xffffffffLL) return SPMM_ERR_INVALID_VALUE;  // rows of B < 4 GiB apart
-    SddmmArgs a{m, n, nnz, row_ptr, col_ind, dC, lddc, B, ldb, out, 32, k};
+    SddmmArgs a{m, n, nnz, row_ptr, col_ind, dC, lddc, B, ldb, out, 32};
     cudaStream_t s = (cudaStream_t)stream;
     if (n == 0) {  // empty dot products
         const int es = out_type == SPMM_F32 ? 4 : 2;
         return status_of(cudaMemsetAsync(out, 0, (size_t)nnz * es, s));
     }
-    if (b_type == SPMM_F32 && out_type == SPMM_F32) return sddmm_run<float, float>(a, s);
-    if (b_type == SPMM_BF16 && out_type == SPMM_BF16) return sddmm_run<__nv_bfloat16, __nv_bfloat16>(a, s);
-    if (b_type == SPMM_BF16 && out_type == SPMM_F32) return sddmm_run<__nv_bfloat16, float>(a, s);
-    if (b_type == SPMM_F16 && out_type == SPMM_F16) return sddmm_run<__half, __half>(a, s);
-    if (b_type == SPMM_F16 && out_type == SPMM_F32) return sddmm_run<__half, float>(a, s);
+    if (b_type == SPMM_F32 && out_type == SPMM_F32) return sddmm_run<float, float>(a, k, s);
+    if (b_type == SPMM_BF16 && out_type == SPMM_BF16) return sddmm_run<__nv_bfloat16, __nv_bfloat16>(a, k, s);
+    if (b_type == SPMM_BF16 && out_type == SPMM_F32) return sddmm_run<__nv_bfloat16, float>(a, k, s);
+    if (b_type == SPMM_F16 && out_type == SPMM_F16) return sddmm_run<__half, __half>(a, k, s);
+    if (b_type == SPMM_F16 && out_type == SPMM_F32) return sddmm_run<__half, float>(a, k, s);
     return SPMM_ERR_UNSUPPORTED;
 }
 
