@@ -85,7 +85,8 @@ __global__ void __launch_bounds__(kMergeThreads, merge_min_blocks<TB, VEC, E, W>
     bool col_ok[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) col_ok[e] = col0 + e * W * VEC < a.n;
-    const TB* const b_col = B + (col_ok[0] ? col0 : 0);  // row 0 of B; lanes past n read along with column 0
+    // row 0 of B; lanes past n read along with the slab's first column, which the warp reads anyway
+    const TB* const b_col = B + (col_ok[0] ? col0 : (int)blockIdx.y * (W * VEC * E));
     const unsigned ldb_bytes = (unsigned)(a.ldb * (long long)sizeof(TB));
 
     int mc;
