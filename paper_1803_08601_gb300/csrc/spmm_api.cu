@@ -469,7 +469,7 @@ HybridLayout hybrid_layout(int m, long long nnz, int n, const Shape& s, const sp
     H.seg_len = 16 * (32 / s.W) * bs;
     if (t.block_rows > 0) {
         H.block_rows = std::min(t.block_rows, kMaxBlockRows);
-    } else if (s.W * s.vec > 32 || s.slabs > 1) {
+    } else if (s.W * s.vec > 32 || (s.vec > 1 && s.slabs > 1)) {
         H.block_rows = s.W >= 16 ? 64 : 128;
     } else {  // whole waves of the row-block pass's resident warps (3 or 4 CTAs of 8 per SM)
         const long long base = s.W >= 16 ? 64 : 128, wave = (s.W >= 16 ? 3LL : 4LL) * 8 * 152;
