@@ -178,13 +178,15 @@ int spmm_select_alg_gb300(int m, long long nnz, long long max_row_len, int n, in
  * kernel has overtaken since the sweeps, unless n > 1 and one of these holds, with
  * rows of B in whole 16-byte vectors:
  *   - a Type 1 matrix, rows of B of at most 64 bytes and 6 million nonzeros, or of
- *     at most 128 bytes in 16 bits and 4 million (not whole vectors: n = 2 and 12
- *     million);
- *   - otherwise, rows of B of at most 128 bytes and 1.5 million nonzeros (1 million
- *     where d < 2.25); of at most 256 in 16 bits and 300,000 (any number where
- *     d < 2.25); of at most 256 in 32 bits and 1.5 million (450,000 where d < 2.25,
- *     1.1 million for 256 bytes); of 512 bytes or more (in 16 bits, below 640) and
- *     520,000 rows.
+ *     at most 128 bytes in 16 bits and 4 million, 2^23 where d >= 40 (not whole
+ *     vectors: n = 2, 12 million and d < 40);
+ *   - otherwise, rows of B of at most 128 bytes and 1.4 million nonzeros (900,000
+ *     where d < 2.25); of at most 256 in 16 bits, 300,000 (40,000 where d < 2.25) and
+ *     a longest row of at most 64; of at most 256 in 32 bits and 1.5 million (450,000
+ *     where d < 2.25, 1.1 million for 256 bytes); of 512 bytes or more (in 16 bits,
+ *     below 640) and 520,000 rows.
+ * A call whose B or C is not aligned to whole vectors (pointer, leading dimension)
+ * runs merge in the hybrid's place too, for n > 2.
  * A call that is lent too small a workspace for merge, but one that
  * the hybrid fits, runs the hybrid.
  */

@@ -714,6 +714,9 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
         return cuda_status(L->tiled(ta, shape, s));
     }
     if (a == SPMM_ALG_ROW_SPLIT_HYBRID) {
+        if (alg == SPMM_ALG_ROW_SPLIT_HYBRID && n > 2 &&  // unaligned rows of B or C: element by element
+            !access_ok(16 / dtype_size(b_type), n, b_type, c_type, B, ldb, C, ldc))
+            alg = SPMM_ALG_MERGE;
         const HybridLayout H = hybrid_layout(m, nnz, n, shape, t_eff);
         bool own = false;
         unsigned char* ws = static_cast<unsigned char*>(workspace);
@@ -887,11 +890,13 @@ int spmm_select_alg_gb300(int m, long long nnz, long long max_row_len, int n, in
 // on GB300, hybrid / merge (us).  Power-law rows: 5.3M nonzeros, bf16 n = 16
 // 92 / 87, n = 64 157 / 178; 6.7M, n = 8 74 / 82, n = 32 120 / 109, bf16 n = 64
 // 165 / 214; 23.5M, n = 2 162 / 181, n = 8 177 / 228, n = 20 and up, 20 % behind;
-// 1.9M, everything behind.  Fewer than 3 per row: 1.2M rows of 2, n = 32 87 / 95,
+// 33M of mean 68, n = 4, 220 / 335, 7.3M of mean 70, n = 16, 93 / 82; 1.9M,
+// everything behind.  Fewer than 3 per row: 1.2M rows of 2, n = 32 87 / 95,
 // n = 40 1.18 times, n = 64 150 / 160, n = 128 283 / 301, n = 100 1.3 behind;
-// 500,000 rows of 1, n = 40 52 / 59, n = 64 0.92 times, bf16 n = 128 68 / 87;
-// bf16 n = 256, 800,000 of 1, 150 / 229, and 500,000 0.82 times.  With n = 1 merge
-// is the SpMV kernel, the hybrid one lane per row: 1M power law, 124 / 94.
+// 500,000 rows of 1, n = 40 52 / 59, n = 64 0.92 times, bf16 n = 128 68 / 87, but
+// 7,000 of up to 450 74 / 24; bf16 n = 256, 800,000 of 1, 150 / 229, and 500,000
+// 0.82 times.  With n = 1 merge is the SpMV kernel, the hybrid one lane per row:
+// 1M power law, 124 / 94.
 int spmm_auto_gb300_alg(int m, long long nnz, long long max_row_len, int n, int b_type) {
     const int a = spmm_select_alg_gb300(m, nnz, max_row_len, n, b_type);
     if (a != SPMM_ALG_ROW_SPLIT_HYBRID) return a;
@@ -900,10 +905,11 @@ int spmm_auto_gb300_alg(int m, long long nnz, long long max_row_len, int n, int 
     const bool type1 = max_row_len > 1024 && max_row_len * 8192 >= nnz;
     const bool shortest = nnz * 4 < m * 9LL;  // below 2.25 nonzeros per row
     bool ahead = false;
-    if (row_bytes % 16 != 0) ahead = type1 && n == 2 && nnz >= 12000000;
-    else if (type1) ahead = row_bytes <= 64 ? nnz >= 6000000 : elem == 2 && nnz >= 4000000;
-    else if (row_bytes <= 128) ahead = nnz >= (shortest ? 1000000 : 1500000);
-    else if (row_bytes <= 256 && elem == 2) ahead = shortest || nnz >= 300000;
+    if (row_bytes % 16 != 0) ahead = type1 && n == 2 && nnz >= 12000000 && nnz < 40LL * m;
+    else if (type1 && nnz >= 40LL * m) ahead = nnz >= (8LL << 20) && (row_bytes <= 64 || elem == 2);
+    else if (type1) ahead = nnz >= (row_bytes <= 64 ? 6000000 : 4000000) && (row_bytes <= 64 || elem == 2);
+    else if (row_bytes <= 128) ahead = nnz >= (shortest ? 900000 : 1400000);
+    else if (row_bytes <= 256 && elem == 2) ahead = max_row_len <= 64 && nnz >= (shortest ? 40000 : 300000);
     else if (row_bytes <= 256) ahead = nnz >= (!shortest ? 1500000 : row_bytes < 256 ? 450000 : 1100000);
     else if (row_bytes >= 512) ahead = m >= 520000 && (elem == 4 || row_bytes < 640);
     return ahead ? a : (int)SPMM_ALG_MERGE;
