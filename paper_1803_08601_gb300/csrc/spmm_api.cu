@@ -759,7 +759,12 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
         if (spmv)
             return cuda_status(
                 L->spmv_rowsplit(ra, t_eff.lanes_per_row > 0 ? t_eff.lanes_per_row : spmv_lanes(m, nnz), s));
-        if (shape.vec == 1) shape = unaligned_shape(shape, n, b_type, c_type, B, ldb, C, ldc, tuning);
+        // One pass over up to 128 columns makes a long row's walk longer.  Where the longest row is known to be
+        // what the call waits for, or the rows are too few to fill the GPU, a row's columns stay with as many
+        // warps as there are passes of 32 (power law, longest row 2600, n = 94: 130 us, in one pass 290).
+        const bool long_walk = n <= 128 && (dtype_size(b_type) == 4 ? n > 64 : !access_ok(2, n, b_type, c_type, B, ldb, C, ldc));
+        const bool waits = m <= 8 * 152 || (lmax > 64 && lmax * m > 8 * nnz);
+        if (shape.vec == 1 && !(long_walk && waits)) shape = unaligned_shape(shape, n, b_type, c_type, B, ldb, C, ldc, tuning);
         return cuda_status(L->rowsplit(ra, shape, s));
     }
 
