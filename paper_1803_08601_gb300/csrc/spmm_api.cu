@@ -189,10 +189,15 @@ bool hybrid_two_vectors(int n, int b_type, long long ldb, long long ldc, const S
 // / 1.36 / 1.35; 900,000 rows of B: 3 pieces 0.82 / 0.87 / 0.90, 4 0.97 / 1.04 /
 // 1.08, 6 0.85 / 1.00 / 1.05; 2M rows with one nonzero each, 4 pieces 1.06; bf16,
 // 900,000 rows: 4 pieces 0.86 / 0.95 / 1.01, 8 0.88 / 0.94 / 1.02, 16 0.94 / 1.03
-// / 1.14.
-bool narrow_slabs_pay(long long pieces, long long width, double lanes_used, int m, int k, long long nnz, int elem,
-                      long long l2) {
+// / 1.14.  Rows of A below 5.5 nonzeros (8 for many pieces) pay the passes without
+// the gain (315,000 of 2.1, n = 116, 99 -> 132 us), and slabs of rows that are not
+// whole 128-byte lines touch more of them (790,000 of 13, n = 64, ldb = 68, 388 ->
+// 486), unless the wide passes leave many lanes idle.
+bool narrow_slabs_pay(long long pieces, long long width, long long stride, double lanes_used, int m, int k,
+                      long long nnz, int elem, long long l2) {
     const double d = (double)nnz / m, slab = (double)k * width / l2;
+    if (d < (pieces > 4 ? 8.0 : 5.5)) return false;
+    if (stride % 128 != 0 && (lanes_used > 0.72 || slab > 2.0 / 3)) return false;  // slabs of parts of lines
     const bool idle = lanes_used <= 0.875, rare = nnz < 4LL * k;
     // long rows, too few of them to fill the GPU with more passes
     if (d >= 64 && rare && m * pieces < (elem == 2 ? 20000 : 40000) && !(idle && elem == 2)) return false;
@@ -225,8 +230,9 @@ bool narrow_slabs_pay(long long pieces, long long width, double lanes_used, int 
 // narrower rows lose).  Merge rows of 512 bytes stay whole below 3 nonzeros per
 // row of A, where half-rows pay for another walk and for the sum over two lane
 // groups at every row end: 900,000 rows of 1, bf16 n = 256, 265 -> 165 us; of
-// Poisson 1.3, float32 n = 128, 194 -> 181.
-int default_slabs(int alg, int m, int k, long long nnz, int n, int b_type, bool plus_times) {
+// Poisson 1.3, float32 n = 128, 194 -> 181.  16-bit rows of 256 bytes go to the
+// narrow kernel in halves below 2.5: 1.2M of 1, bf16 n = 128, 176 -> 131.
+int default_slabs(int alg, int m, int k, long long nnz, int n, int b_type, long long ldb, bool plus_times) {
     static std::atomic<int> l2_cache[64];  // 0 until first queried; every thread stores the same value
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 1;
@@ -248,7 +254,7 @@ int default_slabs(int alg, int m, int k, long long nnz, int n, int b_type, bool 
         for (long long w = width; w >= 128; w /= 2) {
             const long long pieces = (row_bytes + w - 1) / w;
             if (pieces * w * 7 > row_bytes * 8) continue;
-            if (!narrow_slabs_pay(pieces, w, used, m, k, nnz, elem, l2)) break;
+            if (!narrow_slabs_pay(pieces, w, ldb * elem, used, m, k, nnz, elem, l2)) break;
             return (int)std::min<long long>(pieces, 65535);
         }
     }
@@ -704,7 +710,7 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
     }
     const int a = resolve_alg(alg, m, nnz, tuning);
     spmm_tuning_t t_eff = tuning ? *tuning : spmm_tuning_t{};
-    if (t_eff.column_slabs <= 0 && t_eff.lanes_per_row <= 0) t_eff.column_slabs = default_slabs(a, m, k, nnz, n, b_type, L->plus_times);
+    if (t_eff.column_slabs <= 0 && t_eff.lanes_per_row <= 0) t_eff.column_slabs = default_slabs(a, m, k, nnz, n, b_type, ldb, L->plus_times);
     if (!choose_shape(n, b_type, c_type, B, ldb, C, ldc, &t_eff, &shape)) return SPMM_ERR_INVALID_VALUE;
     if (a == SPMM_ALG_ROW_SPLIT_HYBRID && hybrid_two_vectors(n, b_type, ldb, ldc, shape) && !shape_for(n, 8, &t_eff, &shape))
         return SPMM_ERR_INVALID_VALUE;
@@ -930,7 +936,7 @@ double spmm_tiled_reuse(int m, int k, long long nnz, int n, int b_type) {
 
 int spmm_default_column_slabs(int alg, int k, int n, int b_type) {
     if (k < 0 || n < 0 || dtype_size(b_type) == 0) return 1;
-    return spmm::default_slabs(alg, k, k, 8LL * k, n, b_type, true);  // k rows of 8
+    return spmm::default_slabs(alg, k, k, 8LL * k, n, b_type, 128, true);  // k rows of 8, in whole lines
 }
 
 int spmm_csr_max_row_length(int m, const int* row_ptr, long long* max_row_len, void* stream) {
