@@ -245,7 +245,8 @@ int default_slabs(int alg, int m, int k, long long nnz, int n, int b_type, long 
     const long long row_bytes = (long long)n * elem;
     const long long min_row = alg == SPMM_ALG_MERGE ? 512 : 256;
     int wide = (long long)k * row_bytes > 2LL * l2 && row_bytes >= min_row ? 2 : 1;
-    if (alg == SPMM_ALG_MERGE && row_bytes <= 512 && nnz < 3LL * m) wide = 1;
+    if (alg == SPMM_ALG_MERGE && row_bytes <= 512 && nnz < 3LL * m)
+        wide = elem == 2 && row_bytes == 256 && 2 * nnz < 5LL * m ? 2 : 1;
     if (alg == SPMM_ALG_ROW_SPLIT && row_bytes >= (plus_times ? 256 : 512) &&
         (long long)k * std::min(row_bytes, 512LL) > l2 / 2) {
         const long long vecs = (row_bytes + 15) / 16, lanes = pow2_ceil((vecs + wide - 1) / wide);
