@@ -602,7 +602,7 @@ __device__ __forceinline__ void merge_kernel_body(const MergeArgs& a) {
     }
 }
 
-// Narrow rows (W <= 8): six CTAs per SM.  Wider ones, and narrow ones of longer
+// Narrow rows (W <= 16): six CTAs per SM.  Wider ones, and narrow ones of longer
 // rows, run merge_kernel (merge.cuh); merge_narrow (spmm_api.cu) has the line.
 template <typename TV, typename TB, typename TC, int VEC, int W, typename SR = PlusTimes>
 __global__ void __launch_bounds__(kNarrowThreads, 6) merge_kernel_narrow(MergeArgs a) {

@@ -229,6 +229,7 @@ cudaError_t merge_narrow_launch(const MergeArgs& a, const Shape& s, int grid_cap
         case 2: return merge_narrow_launch_one<TV, TB, TC, VEC, 2, SR>(a, s, grid_cap, st);
         case 4: return merge_narrow_launch_one<TV, TB, TC, VEC, 4, SR>(a, s, grid_cap, st);
         case 8: return merge_narrow_launch_one<TV, TB, TC, VEC, 8, SR>(a, s, grid_cap, st);
+        case 16: return merge_narrow_launch_one<TV, TB, TC, VEC, 16, SR>(a, s, grid_cap, st);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -404,7 +405,8 @@ size_t merge_smem_vec(const Shape& s) {
         case 1: return MergeSmem<TV, VEC, 1, kNarrowThreads>::total(s.ips);
         case 2: return MergeSmem<TV, VEC, 2, kNarrowThreads>::total(s.ips);
         case 4: return MergeSmem<TV, VEC, 4, kNarrowThreads>::total(s.ips);
-        default: return MergeSmem<TV, VEC, 8, kNarrowThreads>::total(s.ips);
+        case 8: return MergeSmem<TV, VEC, 8, kNarrowThreads>::total(s.ips);
+        default: return MergeSmem<TV, VEC, 16, kNarrowThreads>::total(s.ips);
     }
 }
 

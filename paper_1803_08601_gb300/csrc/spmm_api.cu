@@ -296,15 +296,21 @@ MergeLayout merge_layout(long long num_tiles, int warps, int n) {
 // tile together) for column slabs of shape s.  With W lanes per row the warp
 // adds up 32 / W lane groups' partial sums at every row end, which short rows
 // do not repay: up to 4 lanes of 16 bytes, 8 lanes below a mean of 4 nonzeros
-// per row, and unaligned rows of up to 4 columns below 8 and of up to 8 below
-// 3.5 run the narrow kernel.
+// per row, and 16 below 1.2 (2.2 with many) run the narrow kernel.  In 16 bits 8
+// lanes do so further up, where the conversions that a warp makes one nonzero at
+// a time bind, and unaligned rows of W lanes up to the means below.
 // Measured on GB300, narrow / the other (us): 300,000 rows of Poisson 8,
 // n = 16, 41 / 51; 400,000 of Poisson 2.5, n = 32, 42 / 46; 700,000 of Poisson
-// 5, n = 32, 94 / 88; 700,000 of Poisson 5, n = 2, 43 / 55;
-// 500,000 of Poisson 3, n = 5, 48 / 57, 1M of Poisson 4, 93 / 91.
+// 5, n = 32, 94 / 88; 1.2M of 1, n = 48, 103 / 121; bf16
+// n = 64, 3M nonzeros of mean 5 0.65 times, of 12 0.9, of 40 1.12, 10M of any 0.8;
+// 380,000 of 15, n = 2, 46 / 68; 500,000 of Poisson 3, n = 5, 48 / 57, 1M of
+// Poisson 4, 93 / 91.
 bool merge_narrow(int m, long long nnz, const Shape& s) {
+    if (s.vec == 8 && s.W == 8) return nnz >= 8000000 || nnz < (nnz >= 2500000 ? 30LL : 8LL) * m;
+    if (s.W == 16) return s.vec == 1 ? 20 * nnz <= 21LL * m : 10 * nnz < (nnz >= 1100000 ? 22LL : 12LL) * m;
     if (s.vec > 1) return s.W <= 4 || (s.W == 8 && nnz < 4LL * m);
-    return s.W <= 4 ? nnz < 8LL * m : s.W == 8 && 2 * nnz < 7LL * m;
+    if (s.W <= 2) return nnz < (nnz >= 800000 ? 26LL : 8LL) * m;
+    return s.W <= 4 ? nnz < 9LL * m : s.W == 8 && 2 * nnz < 7LL * m;
 }
 
 // Lane layout where 16-byte accesses are not aligned (base.vec == 1): up to 128
@@ -344,17 +350,18 @@ MergeLayout merge_layout(int m, long long nnz, int n, const MergeTiles& t) {
 //
 // merge_kernel_narrow: tiles of kNarrowTile items, or smaller ones that make one
 // or two whole waves of its persistent CTAs (6 per SM) where kNarrowTile would
-// make at most two.  400,000 rows of Poisson 2.5, n = 32: 1.5 waves of 1024
-// items 47 us, 2 of 768 42 us.
+// make at most one or two.  400,000 rows of Poisson 2.5, n = 32: 1.5 waves of 1024
+// items 47 us, 2 of 768 42 us; 13,500 of 63, n = 4: one of 948 18, two of 474 21.
 constexpr long long kNarrowWave = 6 * 152;
 long long narrow_tiles(long long total) {
     if (total >= 2 * kNarrowWave * kNarrowTile) return (total + kNarrowTile - 1) / kNarrowTile;
-    return std::min((total + 127) / 128, (total < kNarrowWave * kNarrowTile * 5 / 8 ? 1 : 2) * kNarrowWave);
+    return std::min((total + 127) / 128, (total <= kNarrowWave * kNarrowTile ? 1 : 2) * kNarrowWave);
 }
 
 // merge_kernel: a warp takes about kMergeTile items, so that the tiles make whole
-// waves of the warps that the GPU runs at once (28 or 32 per SM): a wave filled
-// to a tenth costs as much as a full one.  300,000 rows of Poisson 8, n = 128:
+// waves of the warps that the GPU runs at once: 28 (W < 32) or 32 per SM with
+// 16-byte accesses; up to 40 with narrower ones, which fill 0.7 or 0.8 of a wave.
+// A wave filled to a tenth costs as much as a full one.  300,000 rows of Poisson 8, n = 128:
 // 1.08 waves of 512 items 190 us, one wave of 555 147 us.
 constexpr int kMergeTile = 512;
 long long warp_wave(int W) { return (W < 32 ? 28LL : 32LL) * 152; }
@@ -375,7 +382,7 @@ long long full_tile(const spmm_tuning_t* t, const Shape& shape, int sv) {
         if (sv == 4) return s.vec == 1 ? merge_smem_vec<float, 1>(s) : s.vec == 4 ? merge_smem_vec<float, 4>(s) : merge_smem_vec<float, 8>(s);
         return s.vec == 1 ? merge_smem_vec<__half, 1>(s) : s.vec == 4 ? merge_smem_vec<__half, 4>(s) : merge_smem_vec<__half, 8>(s);
     };
-    while (s.W <= 8 && s.ips > 4 && smem() > kMaxSmem) s.ips = s.ips * 3 / 4;
+    while (s.W <= 16 && s.ips > 4 && smem() > kMaxSmem) s.ips = s.ips * 3 / 4;
     return (long long)groups * s.ips;
 }
 
@@ -436,7 +443,7 @@ size_t merge_bound(int m, long long nnz, int n, const spmm_tuning_t* t, const Sh
     const long long quarter = (full + kMergeWarps - 1) / kMergeWarps;
     const size_t full_bytes = full_tiles_bytes(m, nnz, n, t, s, 4);
     size_t tiled = merge_layout(asked ? (total + quarter - 1) / quarter : warp_tiles(total, s.W), kMergeWarps, n).total;
-    if (s.W <= 8) tiled = std::max(tiled, merge_layout(asked ? (total + full - 1) / full : narrow_tiles(total), 1, n).total);
+    if (s.W <= 16) tiled = std::max(tiled, merge_layout(asked ? (total + full - 1) / full : narrow_tiles(total), 1, n).total);
     const size_t most = std::max(full_bytes, std::min<size_t>(full_bytes / 4 * 15, 8u << 20));
     return align256(std::max(full_bytes, std::min(tiled, most)));
 }
@@ -707,6 +714,9 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
     bool for_hybrid = false;  // merge in the place of the hybrid that the selector names
     if (alg == SPMM_ALG_AUTO_GB300) {
         alg = spmm_auto_gb300_alg(m, nnz, lmax, n, b_type);
+        if (alg == SPMM_ALG_ROW_SPLIT_HYBRID && n > 2 &&  // unaligned rows of B or C: element by element
+            !access_ok(16 / dtype_size(b_type), n, b_type, c_type, B, ldb, C, ldc))
+            alg = SPMM_ALG_MERGE;
         for_hybrid = alg == SPMM_ALG_MERGE && spmm_select_alg_gb300(m, nnz, lmax, n, b_type) == SPMM_ALG_ROW_SPLIT_HYBRID;
     }
     const int a = resolve_alg(alg, m, nnz, tuning);
@@ -721,9 +731,6 @@ int run_spmm(const Launchers* L, int m, int k, int n, long long nnz, const int* 
         return cuda_status(L->tiled(ta, shape, s));
     }
     if (a == SPMM_ALG_ROW_SPLIT_HYBRID) {
-        if (alg == SPMM_ALG_ROW_SPLIT_HYBRID && n > 2 &&  // unaligned rows of B or C: element by element
-            !access_ok(16 / dtype_size(b_type), n, b_type, c_type, B, ldb, C, ldc))
-            alg = SPMM_ALG_MERGE;
         const HybridLayout H = hybrid_layout(m, nnz, n, shape, t_eff);
         bool own = false;
         unsigned char* ws = static_cast<unsigned char*>(workspace);

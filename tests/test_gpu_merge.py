@@ -102,3 +102,27 @@ def test_unaligned_short_rows_are_bitwise(gpu_lib, n, mean):
     for tuning in (None, dict(column_slabs=2), dict(items_per_subwarp=5)):
         C = gpu_lib.spmm(d_rp, d_ci, d_v, d_B, alg="merge", nnz=int(rp[-1]), tuning=tuning)
         assert np.array_equal(C.cpu().numpy(), ref), tuning
+
+
+@pytest.mark.parametrize("n,storage,mean,m", [(12, "float32", 1, 5000), (36, "float32", 1, 5000), (48, "float32", 1, 5000),
+                                              (64, "float32", 1, 9000), (64, "float32", 2, 600_000), (64, "bfloat16", 7, 5000),
+                                              (40, "float16", 9, 5000), (64, "bfloat16", 12, 250_000), (72, "bfloat16", 1, 5000),
+                                              (128, "bfloat16", 1, 5000), (128, "bfloat16", 2, 5000), (2, "float32", 15, 60_000),
+                                              (4, "float32", 60, 14_000)])
+def test_the_lines_of_the_narrow_kernel(gpu_lib, n, storage, mean, m):
+    """Mean row lengths at which rows of 2 to 16 lanes change their kernel, with one long row and empty ones."""
+    import torch
+
+    dt = getattr(torch, storage)
+    g = torch.Generator(device="cuda").manual_seed(n + m)
+    lens = torch.full((m,), mean, dtype=torch.int64, device="cuda")
+    if mean > 1:
+        lens[::50], lens[7], lens[100:180], lens[-3:] = 2 * mean, 700, 0, 0
+    rp = torch.zeros(m + 1, dtype=torch.int32, device="cuda")
+    rp[1:] = torch.cumsum(lens, 0)
+    nnz = int(rp[-1])
+    ci = torch.randint(3000, (nnz,), device="cuda", generator=g).int()
+    v = torch.randint(-2, 3, (nnz,), device="cuda", generator=g).to(dt)
+    B = torch.randint(-3, 4, (3000, n), device="cuda", generator=g).to(dt)
+    C = gpu_lib.spmm(rp, ci, v, B, alg="merge", out_dtype=torch.float32, nnz=nnz)
+    assert torch.equal(C, gpu_lib.spmm(rp, ci, v, B, alg="row_split", out_dtype=torch.float32, nnz=nnz))
