@@ -171,7 +171,9 @@ __device__ __forceinline__ void block_scan2(int& a, int& b, int (*warp_sum)[kRad
 // time took three barriers for every 256 elements, and __match_any_sync in the
 // place of the ballots a third longer.)  Element order is kept among equal
 // digits.  10M keys of 7 bits: 0.12 -> 0.088 ms, the transpose 0.55 -> 0.36.
-// payload_in == nullptr means the payload is the element's own index.
+// payload_in == nullptr means the payload is the element's own index.  Four CTAs
+// per SM leave 64 registers, which hold all but 17 words of a thread's keys and
+// ranks.
 __global__ void __launch_bounds__(kSortThreads, 4) radix_scatter_kernel(
     const int* __restrict__ keys_in, const int* __restrict__ payload_in, long long n, int shift, int mask, int tiles,
     const int* __restrict__ offsets, const int* __restrict__ totals, int* __restrict__ keys_out,
@@ -597,7 +599,8 @@ __global__ void __launch_bounds__(128, sddmm_min_blocks<VEC, E>()) sddmm_warp_ke
 template <typename TD, typename TO, int VEC, int E>
 cudaError_t sddmm_warp_launch(const SddmmArgs& a0, cudaStream_t st, int k = 0) {
     SddmmArgs a = a0;
-    // nonzeros per warp: about 256, in whole waves of the 32 warps that an SM runs at once
+    // nonzeros per warp: about 256, in whole waves of the 32 warps that an SM runs at once (up to 16
+    // columns of dC per lane; the wider layouts run 16 or 8, and two or four waves for one)
     const long long wave = 256LL * 32 * 152, waves = std::max<long long>(1, (a.nnz + wave / 2) / wave);
     const long long per_warp = (a.nnz + waves * 32 * 152 - 1) / (waves * 32 * 152);
     a.chunk = (int)std::max<long long>(32, (per_warp + 31) / 32 * 32);
@@ -634,6 +637,8 @@ cudaError_t sddmm_warp_launch(const SddmmArgs& a0, cudaStream_t st, int k = 0) {
     return cudaSuccess;
 }
 
+// W: up to 8 lanes for the narrow and short rows that sddmm_run leaves to the lane
+// groups, 32 for the wide ones with 16-bit results.
 template <typename TD, typename TO, int VEC>
 cudaError_t sddmm_launch_vec(const SddmmArgs& a, int W, long long groups, cudaStream_t st) {
     const long long blocks = (groups * W + kThreads - 1) / kThreads;
@@ -643,8 +648,12 @@ cudaError_t sddmm_launch_vec(const SddmmArgs& a, int W, long long groups, cudaSt
         case 2: sddmm_kernel<TD, TO, VEC, 2><<<(unsigned)blocks, kThreads, 0, st>>>(a); break;
         case 4: sddmm_kernel<TD, TO, VEC, 4><<<(unsigned)blocks, kThreads, 0, st>>>(a); break;
         case 8: sddmm_kernel<TD, TO, VEC, 8><<<(unsigned)blocks, kThreads, 0, st>>>(a); break;
-        case 16: sddmm_kernel<TD, TO, VEC, 16><<<(unsigned)blocks, kThreads, 0, st>>>(a); break;
-        default: sddmm_kernel<TD, TO, VEC, 32><<<(unsigned)blocks, kThreads, 0, st>>>(a); break;
+        default:
+            if constexpr (sizeof(TO) == 2) {
+                sddmm_kernel<TD, TO, VEC, 32><<<(unsigned)blocks, kThreads, 0, st>>>(a);
+                break;
+            }
+            return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }

@@ -216,10 +216,10 @@ struct MergeArgs {
     int num_tiles;
     int slabs;            // column slabs; work item = slab * num_tiles + tile
     int ips;              // merge-path items per lane group
-    float* carry;         // [num_tiles][n] partial sum of the row a tile leaves unfinished
-    float* head;          // [num_tiles][n] partial sum of the row a tile finishes but did not start
-    int* carry_row;       // [num_tiles] that row, or -1
-    int* head_row;        // [num_tiles] that row, or -1
+    float* carry;         // [CTAs][n] partial sum of the row that a CTA's tiles leave unfinished
+    float* head;          // [CTAs][n] partial sum of the row that they finish but did not start
+    int* carry_row;       // [CTAs] that row, or -1
+    int* head_row;        // [CTAs] that row, or -1
     int* status;          // optional device status word
     int use_tma;          // 1: 1-D bulk copies into shared memory, 0: cooperative loads
     unsigned long long wait_ns;  // limit of every mbarrier wait

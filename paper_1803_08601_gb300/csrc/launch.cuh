@@ -12,11 +12,12 @@
 
 namespace spmm {
 
-// Launch shape chosen by the host: vec = elements per lane access (1 or the
-// 16-byte width of B's type; merge based: any power of two up to it), W =
-// lanes per row, chunks = column chunks of W * vec columns that a lane group
-// covers together (merge based; 1 elsewhere), slabs = column slabs, ips =
-// merge-path items per lane group of merge_kernel_narrow (0: merge_kernel).
+// Launch shape chosen by the host: vec = elements per lane access (the 16-byte
+// width of B's type, or 1 or 2 where that is not aligned; 8 also for float32 in
+// the hybrid), W = lanes per row, chunks = column chunks of W * vec columns that a
+// lane group covers together (merge based and unaligned row split; 1 elsewhere),
+// slabs = column slabs, ips = merge-path items per lane group of
+// merge_kernel_narrow (0: merge_kernel).
 struct Shape {
     int vec;
     int W;

@@ -21,7 +21,9 @@ __host__ __device__ constexpr int merge_unroll() {
 }
 
 // CTAs of 4 warps per SM, as the registers of the gathers in flight and of the
-// row bookkeeping of several lane groups need: 72, 64 or 48 per thread.
+// row bookkeeping of several lane groups need: 72, 64 or 48 per thread.  Up to 12
+// words are spilled where it is 48 (one element per lane and 16 lanes, two and 32)
+// and, in 16 bits, up to 7 of the 16-byte layouts.
 template <typename TB, int VEC, int E, int W>
 __host__ __device__ constexpr int merge_min_blocks() {
     constexpr int bytes = VEC * E * (int)sizeof(TB) * merge_unroll<TB, VEC, E, W>();
