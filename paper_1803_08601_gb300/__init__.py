@@ -313,11 +313,12 @@ def _stream_handle(stream=None) -> int:
     if stream is not None:
         return int(stream.cuda_stream)
     torch = _torch()
-    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
-    if raw is None or device is None or not torch.cuda.is_initialized():
-        return int(torch.cuda.current_stream().cuda_stream)
-    # the handle alone: a Stream object of the current stream costs about 3 us per call
-    return raw(device())
+    if torch.cuda.is_initialized():
+        try:  # the handle alone: a Stream object of the current stream costs about 3 us per call
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        except AttributeError:  # private names, which a torch may not have
+            pass
+    return int(torch.cuda.current_stream().cuda_stream)
 
 
 def _require_cuda(*ts):
