@@ -192,12 +192,15 @@ bool hybrid_two_vectors(int n, int b_type, long long ldb, long long ldc, const S
 // / 1.14.  Rows of A below 5.5 nonzeros (8 for many pieces) pay the passes without
 // the gain (315,000 of 2.1, n = 116, 99 -> 132 us), and slabs of rows that are not
 // whole 128-byte lines touch more of them (790,000 of 13, n = 64, ldb = 68, 388 ->
-// 486), unless the wide passes leave many lanes idle.
+// 486), unless two wide passes or more leave many lanes idle (203,000 of 56, n =
+// 144, 679 -> 435; one that does, 385,000 of 59, n = 84, 795 -> 902).
 bool narrow_slabs_pay(long long pieces, long long width, long long stride, double lanes_used, int m, int k,
                       long long nnz, int elem, long long l2) {
     const double d = (double)nnz / m, slab = (double)k * width / l2;
     if (d < (pieces > 4 ? 8.0 : 5.5)) return false;
-    if (stride % 128 != 0 && (lanes_used > 0.72 || slab > 2.0 / 3)) return false;  // slabs of parts of lines
+    if (stride % 128 != 0 &&  // slabs of parts of lines
+        (pieces * width <= 512 || lanes_used > (elem == 2 ? 0.8 : 0.72) || slab > 2.0 / 3))
+        return false;
     const bool idle = lanes_used <= 0.875, rare = nnz < 4LL * k;
     // long rows, too few of them to fill the GPU with more passes
     if (d >= 64 && rare && m * pieces < (elem == 2 ? 20000 : 40000) && !(idle && elem == 2)) return false;
