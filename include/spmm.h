@@ -209,10 +209,11 @@ double spmm_tiled_reuse(int m, int k, long long nnz, int n, int b_type);
  * these, else one per 128, for rows of 256 bytes or more that the slabs exceed
  * by at most a seventh (semirings other than (+, x): 512 bytes or more).
  * Otherwise 2 when B is larger than twice the L2 and its rows are wide (>= 512
- * bytes for merge, >= 256 bytes otherwise), else 1.  Products of longer rows or
- * of fewer nonzeros per row of B, which narrow slabs do not repay, take the
- * latter number in the place of the former where the slabs are many, and merge
- * leaves rows of 512 bytes whole below 3 nonzeros per row of A.
+ * bytes for merge, >= 256 bytes otherwise), else 1.  Products which narrow slabs do
+ * not repay (longer or shorter rows of A, fewer nonzeros per row of B, rows of B
+ * that are not whole 128-byte lines) take the latter number in the place of the
+ * former.  Below 3 nonzeros per row of A merge leaves rows of 512 bytes whole, and
+ * below 2.5 it halves 16-bit rows of 256.
  * Each slab pass gathers that share of every row of B from a B slab that
  * much smaller.  Reads the L2 size of the current device (no device work).
  * Products whose B and C are not 16-byte aligned take more slabs where a pass
